@@ -41,6 +41,7 @@ struct Plan {
     // state_s: the stored state is s = Lambda_x^{-1} r instead of the weights w
     int G, Gp, ws, threads;
     int rowcache;   // fused kernel: row-table rows a tile may cache in shared memory
+    int nseg;       // fused kernel, FP32: row segments per pair of source columns
     bool full_row, state_s;
     // Galerkin one-pass plan with a separate x pass: tiles without x halo store the deposit into
     // tmp, and a row pass solves Lambda_x along whole rows into the state buffer
@@ -170,17 +171,19 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
         kernel = VP_KERNEL_SCATTER;
     }
     P->G = 8;   // a multiple of 4, so that the x solve's rows start 16-byte aligned
-    P->Gp = 8;
+    // rows: FP32 rings drop rows outside the window in their common path, so four are enough there
+    P->Gp = opts->precision == VP_FP64 ? 8 : 4;
     P->full_row = false;
     P->ws = 0;
     P->threads = 0;
     P->rowcache = 0;
+    P->nseg = 1;
     int ftx = 0, ftp = 0;
     if (kernel == VP_KERNEL_AUTO || kernel == VP_KERNEL_FUSED) {
         const int halo = P->galerkin && !P->xpass ? fused_halo(opts->precision) : 0;
         const int R = basis == VP_BASIS_TENT ? 1 : 2;
         const int G = P->G, Gp = P->Gp;
-        ftx = opts->tile_x ? opts->tile_x : (opts->precision == VP_FP64 ? 128 : 224);
+        ftx = opts->tile_x ? opts->tile_x : (opts->precision == VP_FP64 ? 128 : (halo ? 208 : 240));
         ftp = opts->tile_p ? opts->tile_p : 64;
         bool full = false;
         // whole-period tiles when the mesh is little wider than a windowed tile; by default only
@@ -202,7 +205,15 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
         // two CTAs per SM (up to 320 threads) unless the tile is wide: then one CTA of up
         // to 576 threads per SM
         const bool wide = (wsrc + 31) / 32 * 32 > kFusedThreads2;
-        const int threads = std::min(wide ? kFusedMaxThreads : kFusedThreads2, (wsrc + 31) / 32 * 32);
+        int threads = std::min(wide ? kFusedMaxThreads : kFusedThreads2, (wsrc + 31) / 32 * 32);
+        int nseg = 1;
+        if (sz == 4) {
+            // a thread walks a pair of columns through a segment of the tile's rows: as many segments as
+            // the block's threads serve in one round
+            const int lanes = (wsrc / 2 + 1 + 31) / 32 * 32;
+            nseg = std::max(1, std::min(kFusedThreads32 / lanes, ftp / 8));
+            threads = std::min(kFusedThreads32, lanes * nseg);
+        }
         const size_t cap = wide ? (size_t)200 * 1024 : (size_t)112 * 1024;
         auto smem_of = [&](int tp_) {
             return sz == 8 ? fused_smem_bytes<double>(ws, tp_ + 2 * Gp, threads)
@@ -216,6 +227,7 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
             P->full_row = full;
             P->ws = ws;
             P->threads = threads;
+            P->nseg = nseg;
             // the shared memory left beside the window keeps the tile's row table
             P->rowcache = fused_rowcache_rows(opts->precision, smem, wide ? 1 : 2);
         } else if (kernel == VP_KERNEL_FUSED) {
@@ -430,6 +442,7 @@ FusedArgs<T> fused_args(vp_sim *s, const void *src, void *dst)
     a.hist = s->ptr<double>(P.L.hist);
     a.hist_cap = P.hist_cap;
     a.rowcache = P.rowcache;
+    a.nseg = P.nseg;
     a.xpass = P.xpass ? 1 : 0;
     a.bunch_x = P.xpass && P.fel ? 1.0 / (2.0 / 3.0 + cos(P.g.hx) / 3.0) : 1.0;
     return a;
@@ -1368,7 +1381,7 @@ vp_status vp_batch_create(vp_sim *const *sims, int32_t count, void *stream, void
     {
         // every item runs with the batch's thread count: the row cache takes what is left of
         // the shared memory beside the largest window, if the batch keeps its CTAs per SM
-        const int want = b->threads > kFusedThreads2 ? 1 : 2;
+        const int want = 2;
         int rows = fused_rowcache_rows(VP_FP32, b->smem, want);
         if (rows > 0 && fused_batch_blocks_per_sm(b->basis, b->projection,
                                                   b->smem + (size_t)rows * sizeof(RowEntry<float>),

@@ -12,10 +12,10 @@
 // One CTA owns one destination tile [X0, X0+TX) x [P0, P0+TP). It keeps a
 // shared-memory window: the tile widened by the x-solve halo D and a guard
 // band G. It bounds the source nodes whose pushed B3 footprint reaches the
-// widened tile and gives each thread one source column. The thread walks the
-// column:
+// widened tile. FP32: each thread takes a pair of adjacent source columns through a segment
+// of those rows in packed arithmetic (vp_walk.cuh). FP64: each thread takes one column:
 //   * Galerkin: the p solve is the Thomas algorithm for tridiag(1/6, 2/3, 1/6)
-//     (exact pivots near row 0), walked downwards in chunks of kC rows: the
+//     (exact pivots near row 0), walked downwards in chunks of rows: the
 //     forward sweep of a chunk starts kHalo rows below it (truncation
 //     |z|^kHalo, z = sqrt(3) - 2) and is kept in a shared-memory column buffer;
 //     the back substitution carries on from the chunk above;
@@ -34,6 +34,7 @@
 #include "vp_fel.cuh"
 #include "vp_internal.h"
 #include "vp_sum.cuh"
+#include "vp_walk.cuh"
 
 namespace vp {
 namespace {
@@ -44,13 +45,17 @@ template <typename T>
 struct Halo {
     static constexpr int value = sizeof(T) == 4 ? 16 : 28;
 };
+constexpr int kSumWarps = 8;        // virtual warps of the per-tile FEL column sums
+constexpr int kMinSegRows = 8;      // shortest row segment of the FP32 walk (each restarts its rings)
 constexpr int kC = 16;              // rows per chunk of the p solve (multiple of 4)
-// rows of the per-thread column buffer: one chunk, or the look-ahead above the top row
+// elements of the per-thread column buffer: one chunk of rows, or the look-ahead above the top row;
+// FP32 threads walk two columns
 template <typename T>
 struct GRows {
-    static constexpr int value = kC > Halo<T>::value ? kC : Halo<T>::value;
+    static constexpr int value = sizeof(T) == 4 ? 2 * kC32 : (kC > Halo<T>::value ? kC : Halo<T>::value);
 };
 constexpr int kXBig = kFusedMaxRow / 32;   // elements per lane for rows up to kFusedMaxRow
+constexpr int kXBig32 = 20;                // FP32: whole-period rows of kFusedMaxRow with the halo on both sides
 
 template <typename T, int BASIS>
 struct FTaps;
@@ -66,11 +71,6 @@ struct FTaps<T, VP_BASIS_TENT> {
     }
 };
 
-// FP32: three weights on the grid 2^-23, the fourth one minus them, so that the four sum to
-// exactly one (see node_taps_f32); FP64: the fourth from the other three
-__device__ __forceinline__ float grid23(float x) { return __fadd_rn(__fadd_rn(x, 1.f), -1.f); }
-__device__ __forceinline__ double grid23(double x) { return x; }
-
 template <typename T>
 struct FTaps<T, VP_BASIS_CUBIC_BSPLINE> {
     static constexpr int N = 4;
@@ -82,11 +82,9 @@ struct FTaps<T, VP_BASIS_CUBIC_BSPLINE> {
         const T t2 = t * t, s2 = s * s;
         const T t3 = t2 * t, s3 = s2 * s;
         const T sixth = T(1) / T(6), two3 = T(2) / T(3);
-        w[0] = grid23(s3 * sixth);
-        w[3] = grid23(t3 * sixth);
-        w[1] = grid23(two3 - t2 + T(0.5) * t3);
-        // the weights sum to one: forming w[2] from the formula instead would carry the rounding
-        // of 2/3 (FP32: a mean excess of 4e-8 per axis) into the mass of every step
+        w[0] = s3 * sixth;
+        w[3] = t3 * sixth;
+        w[1] = two3 - t2 + T(0.5) * t3;
         w[2] = ((T(1) - w[0]) - w[3]) - w[1];
     }
 };
@@ -141,10 +139,6 @@ __device__ void sin_range32(float lo, float hi, float &smin, float &smax)
 // native integer shared-memory atomics (a float atomicAdd on shared memory is a
 // compare-and-swap loop) and the sums do not depend on the order of the additions: the
 // FP32 step is bit-reproducible. FP64: doubles.
-__device__ __forceinline__ void wadd(float *p, float v)
-{
-    atomicAdd(reinterpret_cast<int *>(p), __float2int_rn(v));
-}
 __device__ __forceinline__ void wadd(double *p, double v) { atomicAdd(p, v); }
 // raw cell value (in the tile's scaled units)
 __device__ __forceinline__ double wraw(const float *p) { return (double)*reinterpret_cast<const int *>(p); }
@@ -326,21 +320,7 @@ __device__ __forceinline__ void ring_final(T *win, const WinGeom &W, Ring<T, N> 
 
 // floor of x as a value and as an int without float-to-int conversion instructions:
 // adding 1.5 * 2^(mantissa bits) rounds to an integer held in the low mantissa bits
-// (valid for |x| < 2^22 in FP32, 2^51 in FP64); one compare turns rounding into floor.
-__device__ __forceinline__ void floor_split(float x, float &fl, int &i)
-{
-    const float magic = 12582912.0f;   // 1.5 * 2^23
-    const float t = x + magic;
-    float r = t - magic;
-    int k = __float_as_int(t) - 0x4B400000;
-    if (r > x) {
-        r -= 1.0f;
-        k -= 1;
-    }
-    fl = r;
-    i = k;
-}
-
+// (valid for |x| < 2^51); one compare turns rounding into floor.
 __device__ __forceinline__ void floor_split(double x, double &fl, int &i)
 {
     const double magic = 6755399441055744.0;   // 1.5 * 2^52
@@ -361,99 +341,10 @@ struct ColC {
     T uf, vf, cu1, cu2, cv1, cv2;
 };
 
-// FP32 pairs (x half, p half) in one 64-bit register, for packed FADD2 / FMUL2 / FFMA2
-typedef unsigned long long f2_t;
-__device__ __forceinline__ f2_t f2_pack(float a, float b)
-{
-    f2_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void f2_unpack(f2_t r, float &a, float &b)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
-}
-__device__ __forceinline__ f2_t f2_add(f2_t a, f2_t b)
-{
-    f2_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2_t f2_mul(f2_t a, f2_t b)
-{
-    f2_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2_t f2_fma(f2_t a, f2_t b, f2_t c)
-{
-    f2_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
-// FP32 node: push and tap weights of the x and p axes together in packed pairs. The base
-// cell is round(x - 1/2), so the fraction t lies in [0, 1] (t = 1 at an exact node gives
-// the same deposit as t = 0 one cell further: the B3 and tent kernels are continuous).
-// SROW: the row entry lives in shared memory (the tile's row cache), else in global memory
-template <int BASIS, bool UTERM, bool SROW>
-__device__ __forceinline__ void node_taps_f32(const ColC<float> &c, const RowEntry<float> &r,
-                                              int colrel, int rowrel, float w, int &m, int &n,
-                                              float *wx, float *wy)
-{
-    const float4 *rq = reinterpret_cast<const float4 *>(&r);
-    const float4 q0 = SROW ? rq[0] : __ldg(rq);       // ui, vi, uf, vf
-    const float4 q1 = SROW ? rq[1] : __ldg(rq + 1);   // cy, cy, sy, sy
-    f2_t F = f2_add(f2_pack(c.uf, c.vf), f2_pack(q0.z, q0.w));
-    F = f2_fma(f2_pack(UTERM ? c.cu1 : 0.f, c.cv1), f2_pack(q1.x, q1.y), F);
-    F = f2_fma(f2_pack(UTERM ? c.cu2 : 0.f, c.cv2), f2_pack(q1.z, q1.w), F);
-    const f2_t M1 = f2_pack(-1.f, -1.f), ONE = f2_pack(1.f, 1.f);
-    const f2_t MAG = f2_pack(12582912.f, 12582912.f);   // 1.5 * 2^23
-    const f2_t TT = f2_add(f2_add(F, f2_pack(-0.5f, -0.5f)), MAG);
-    const f2_t R = f2_add(TT, f2_pack(-12582912.f, -12582912.f));
-    const f2_t T = f2_fma(R, M1, F);
-    float tu_bits, tv_bits;
-    f2_unpack(TT, tu_bits, tv_bits);
-    const int iu = __float_as_int(tu_bits) - 0x4B400000, iv = __float_as_int(tv_bits) - 0x4B400000;
-    using TP = FTaps<float, BASIS>;
-    m = colrel + c.ui + __float_as_int(q0.x) + iu + TP::LO;
-    n = rowrel + c.vi + __float_as_int(q0.y) + iv + TP::LO;
-    const f2_t S = f2_fma(T, M1, ONE);
-    if (BASIS == VP_BASIS_TENT) {
-        f2_unpack(S, wx[0], wy[0]);
-        f2_unpack(T, wx[1], wy[1]);
-    } else {
-        const f2_t T2 = f2_mul(T, T), S2 = f2_mul(S, S);
-        const f2_t T3 = f2_mul(T2, T), S3 = f2_mul(S2, S);
-        const float sixth = 1.f / 6.f, two3 = 2.f / 3.f;
-        const f2_t SIX = f2_pack(sixth, sixth);
-        // three weights rounded to multiples of 2^-23 ((x + 1) - 1), the fourth 1 minus them:
-        // every step is then exact and the four sum to exactly one, so the step keeps the mass
-        // up to unbiased rounding whatever the fractions (a pushed node at t = 0, as in a slow
-        // or resting flow, would otherwise lose 2^-26 of its weight per axis and step)
-        const f2_t MONE = f2_pack(-1.f, -1.f);
-        const f2_t W0 = f2_add(f2_add(f2_mul(S3, SIX), ONE), MONE);
-        const f2_t W3 = f2_add(f2_add(f2_mul(T3, SIX), ONE), MONE);
-        const f2_t W1 = f2_add(f2_add(f2_fma(T3, f2_pack(0.5f, 0.5f), f2_fma(T2, M1, f2_pack(two3, two3))),
-                                      ONE), MONE);
-        const f2_t W2 = f2_fma(W1, M1, f2_fma(W3, M1, f2_fma(W0, M1, ONE)));
-        f2_unpack(W0, wx[0], wy[0]);
-        f2_unpack(W1, wx[1], wy[1]);
-        f2_unpack(W2, wx[2], wy[2]);
-        f2_unpack(W3, wx[3], wy[3]);
-    }
-#pragma unroll
-    for (int b = 0; b < TP::N; ++b) wy[b] *= w;
-}
-
-template <typename T, int BASIS, bool UTERM, bool SROW>
+template <typename T, int BASIS, bool UTERM>
 __device__ __forceinline__ void node_taps(const ColC<T> &c, const RowEntry<T> &r, int colrel,
                                           int rowrel, T w, int &m, int &n, T *wx, T *wy)
 {
-    if constexpr (sizeof(T) == 4) {
-        node_taps_f32<BASIS, UTERM, SROW>(c, r, colrel, rowrel, w, m, n, wx, wy);
-        return;
-    }
     using TP = FTaps<T, BASIS>;
     T fu = c.uf + r.uf;
     if (UTERM) fu += c.cu1 * r.cy + c.cu2 * r.sy;
@@ -799,6 +690,78 @@ __device__ __forceinline__ void gal_rows(T *win, const WinGeom &W, T *dst, int L
     }
 }
 
+// FP32: Lambda_x solve of the tile's window rows and the tile store, one warp per row, always as a row of
+// 32 KX elements (every power of z a compile-time constant): the tile's own columns with at least the halo
+// on both sides. Window columns beyond the widened tile hold partial deposits or zeros; what they change in
+// the own columns weighs |z|^17 or less, the truncation of the halo. Whole-period rows take their halo from
+// the period's other end. (A row of another length through run-time chunk lengths cost 2700 cycles against
+// about 300.)
+template <int KX>
+__device__ __forceinline__ void solve_rows_f32(float *win, const WinGeom &W, float *dst, bool full, int G, int Gp, int TXe,
+                                               int TPe, int P0, int X0, int nx, bool want_part, int warp,
+                                               int nwarps, int lane, float sh, float sl, float iq, float &om, bool &bad)
+{
+    constexpr int D = Halo<float>::value;
+    static_assert(KX % 4 == 0, "chunks are read 16 bytes at a time");
+    // element e of the row is window column e + o; the own columns start at element s
+    const int o = full ? 0 : (W.own_c0 + TXe + D <= 32 * KX ? 0 : W.own_c0 - D);
+    const int s = full ? D : W.own_c0 - o;
+    const int base = lane * KX;
+    int w0 = base - D;   // whole period: first column of the lane's chunk, wrapped
+    if (full) w0 = imod(w0, nx);
+    for (int rr = warp; rr < TPe; rr += nwarps) {
+        float *row = win + (size_t)(rr + Gp) * W.ws;
+        float v[KX];
+        if (full) {
+            const int *cell = reinterpret_cast<const int *>(row + G);
+            int c = w0;
+#pragma unroll
+            for (int k = 0; k < KX; ++k) {
+                v[k] = base + k < nx + 2 * D ? (float)cell[c] * iq : 0.f;
+                if (++c == nx) c = 0;
+            }
+        } else {
+            const int4 *r4 = reinterpret_cast<const int4 *>(row + o + base);
+#pragma unroll
+            for (int k4 = 0; k4 < KX / 4; ++k4) {
+                const int4 q = base + o + 4 * k4 < W.ws ? r4[k4] : make_int4(0, 0, 0, 0);
+                v[4 * k4 + 0] = (float)q.x * iq;
+                v[4 * k4 + 1] = (float)q.y * iq;
+                v[4 * k4 + 2] = (float)q.z * iq;
+                v[4 * k4 + 3] = (float)q.w * iq;
+            }
+        }
+        if (want_part) __syncwarp();   // the row is read before any of it is overwritten below
+        solve_row_x_exact<float, KX>(nullptr, lane, v, false, sh, sl);
+        float *dp = dst + (size_t)(P0 + rr) * nx + X0 + base - s;
+        float *keep = row + (full ? G + base - s : o + base);
+        if (base >= s && base + KX <= s + TXe && (reinterpret_cast<uintptr_t>(dp) & 15) == 0) {
+#pragma unroll
+            for (int k = 0; k < KX; k += 4) {
+                const float4 q = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+                *reinterpret_cast<float4 *>(dp + k) = q;
+                om = fmaxf(om, fmaxf(fmaxf(fabsf(q.x), fabsf(q.y)), fmaxf(fabsf(q.z), fabsf(q.w))));
+            }
+            // keep s for the column sums
+            if (want_part)
+#pragma unroll
+                for (int k = 0; k < KX; ++k) keep[k] = v[k];
+        } else if (base < s + TXe && base + KX > s) {
+#pragma unroll
+            for (int k = 0; k < KX; ++k)
+                if (base + k >= s && base + k < s + TXe) {
+                    dp[k] = v[k];
+                    om = fmaxf(om, fabsf(v[k]));
+                    if (want_part) keep[k] = v[k];
+                }
+        }
+        float chk = 0.f;   // v * 0 is 0 for finite values and NaN otherwise
+#pragma unroll
+        for (int k = 0; k < KX; ++k) chk = fmaf(v[k], 0.f, chk);
+        bad |= chk != 0.f;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // One destination tile of one simulation (A may live in shared or global memory).
 template <typename T, int BASIS, bool GAL, bool UTERM>
@@ -812,10 +775,13 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
     T *gcol = win + (size_t)A.ws * (A.tp + 2 * A.Gp);   // [GRows][blockDim] column buffer (Galerkin)
     // row cache: the tile's rows ja .. jb of the push's row table (when they fit)
     RowEntry<T> *rowc = reinterpret_cast<RowEntry<T> *>(gcol + (size_t)GRows<T>::value * blockDim.x);
-    __shared__ int s_ia, s_ib, s_ja, s_jb, s_smax, s_omax, s_cached;
-    __shared__ double s_r4[4][kFusedMaxThreads / 32];
+    __shared__ int s_ia, s_ib, s_ja, s_jb, s_omax;
+    __shared__ double s_part[3][kSumWarps], s_lost[kFusedMaxThreads / 32];
     // Thomas pivots of tridiag(1/6, 2/3, 1/6) in T: entry kPivots holds the limit
+    constexpr int kPv = sizeof(T) == 4 ? kPiv32 : kPivots;
     __shared__ T piv_cp[kPivots + 1], piv_ib[kPivots + 1];
+    __shared__ float2 piv32[kPiv32 + 1];
+    __shared__ WalkWin s_win;
     __shared__ T sig_s[kFusedMaxTileP];   // column-sum weights of Lambda_p^{-1} for the tile rows
 
     const Geometry &g = A.g;
@@ -841,6 +807,10 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
     W.G = G;
     W.full = full;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    // the tile's source rectangle, when an earlier step has left it (asked for first: all that follows
+    // depends on it)
+    const int4 known = A.tile_src ? A.tile_src[tile] : make_int4(kTileSrcUnset, 0, 0, 0);
+    const bool cached = known.x != kTileSrcUnset;
 
     {
         const int nvec = (int)(((size_t)W.WH * W.ws * sizeof(T)) / 16);
@@ -848,21 +818,34 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         for (int k = tid; k < nvec; k += blockDim.x) w4[k] = make_uint4(0, 0, 0, 0);
         for (int k = nvec * (16 / (int)sizeof(T)) + tid; k < W.WH * W.ws; k += blockDim.x) win[k] = T(0);
     }
-    for (int k = tid; k <= kPivots; k += blockDim.x) {
-        piv_cp[k] = (T)A.piv[2 * k];
-        piv_ib[k] = (T)A.piv[2 * k + 1];
+    for (int k = tid; GAL && k <= kPv; k += blockDim.x) {
+        // FP32: rows from kPiv32 on take the limit
+        const int e = k == kPv ? kPivots : k;
+        if (sizeof(T) == 4) {
+            piv32[k] = make_float2((float)A.piv[2 * e + 1], (float)A.piv[2 * e]);
+        } else {
+            piv_cp[k] = (T)A.piv[2 * e];
+            piv_ib[k] = (T)A.piv[2 * e + 1];
+        }
     }
     if (GAL && A.fel_partials)
         for (int k = tid; k < TPe; k += blockDim.x) sig_s[k] = (T)A.sigma[P0 + k];
     if (tid == 0) {
-        const int4 e = A.tile_src ? A.tile_src[tile] : make_int4(kTileSrcUnset, 0, 0, 0);
-        s_cached = e.x != kTileSrcUnset;
-        s_ia = s_cached ? e.x : 0x7fffffff;
-        s_ib = s_cached ? e.y : -0x7fffffff;
-        s_ja = s_cached ? e.z : 0x7fffffff;
-        s_jb = s_cached ? e.w : -0x7fffffff;
-        s_smax = 0;
+        s_ia = s_ja = 0x7fffffff;
+        s_ib = s_jb = -0x7fffffff;
         s_omax = 0;
+        if (sizeof(T) == 4) {
+            s_win.WW = W.WW;
+            s_win.WH = W.WH;
+            s_win.G = G;
+            s_win.WP0 = W.WP0;
+            s_win.own_c0 = full ? 0 : W.own_c0;
+            s_win.own_c1 = full ? W.WW : W.own_c1;
+            s_win.np = np;
+            s_win.nx = nx;
+            s_win.full = full;
+            s_win.edge = (P0 == 0 ? 1 : 0) | (P0 + TPe == np ? 2 : 0);
+        }
     }
     double al = g.alpha0, be = g.beta0, M = g.m0, phi = g.phi0;
     if (g.kind == VP_PUSH_FEL_DKD) {
@@ -871,13 +854,13 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         M = A.state[ST_M];
         phi = A.state[ST_PHI];
     }
-    __syncthreads();
 
     // ---- bound the source nodes whose footprint can reach the widened tile (FP32 with
     //      slack: every magnitude here is below 1e5 cells, where FP32 is exact to 1e-2);
     //      a push that does not change between steps gives the same bounds every step
-    const bool cached = s_cached != 0;
+    int ia = known.x, ib = known.y, ja = known.z, jb = known.w;
     if (!cached) {
+        __syncthreads();
         const float SL = 0.05f;
         const float Mf = (float)M, phif = (float)phi;
         const float EU = fabsf((float)g.KU) * Mf, EV = fabsf((float)g.KV) * Mf;
@@ -950,45 +933,14 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
             atomicMin(&s_ja, my_ja);
             atomicMax(&s_jb, my_jb);
         }
+        __syncthreads();
+        ia = s_ia;
+        ib = s_ib;
+        ja = s_ja;
+        jb = s_jb;
+        if (A.tile_src && tid == 0) A.tile_src[tile] = make_int4(ia, ib, ja, jb);
     }
-    __syncthreads();
-    const int ia = s_ia, ib = s_ib, ja = s_ja, jb = s_jb;
-    if (!cached && A.tile_src && tid == 0) A.tile_src[tile] = make_int4(ia, ib, ja, jb);
     double lost = 0.0;   // in the window's scaled units until the end of the tile
-
-    // ---- FP32: fixed-point scale of the window from max|s| over the rows the walk reads, taken
-    //      from the per-tile maxima the previous step (or vp_set_f) recorded for the state.
-    //      The truncated Thomas solve keeps |w| <= 3 max|s| (forward gain 1/(beta - 1/6) <= 2.2,
-    //      back substitution 1/(1 - c') <= 1.37); a cell sums the B3 taps of the nodes pushed near
-    //      it, about one for an area-preserving flow: 8 times that bound fits in int32.
-    T qs = T(1), iq = T(1);
-    if (sizeof(T) == 4) {
-        float mx = 0.f;
-        if (jb >= ja) {
-            const int r0 = GAL ? max(0, ja - kHalo) : ja, r1 = GAL ? min(np - 1, jb + kHalo) : jb;
-            const int wsrc = min(ib - ia + 1, nx);
-            for (int cidx = tid; cidx < wsrc; cidx += blockDim.x) {
-                const int tc = imod(ia + cidx, nx) / A.tx;
-                for (int tr = r0 / A.tp; tr <= r1 / A.tp; ++tr) mx = fmaxf(mx, A.smax_in[tr * A.ntx + tc]);
-            }
-        }
-        if (mx > 0.f && mx <= 3.0e38f) atomicMax(&s_smax, __float_as_int(mx));
-        if (__syncthreads_or(!(mx <= 3.0e38f))) {
-            qs = T(0);   // a non-finite state, reported when it was written: its deposit is dropped
-            iq = T(0);
-        } else {
-            // the scale is a power of two, so that iq = 1 / qs is exact (a rounded iq scales the
-            // tile's weights by 1 +- 6e-8, a gain that repeats over the steps while the tile's
-            // maximum stays put): qs = 2^(32 - e) with m = f 2^e, f in [0.5, 1), i.e. qs m in
-            // [2^31, 2^32): a cell reaches 2^31 only at 4 to 8 times the largest weight (16 to 32
-            // times with the Thomas gain bound), against about one for an area-preserving flow
-            const float m = fmaxf(__int_as_float(s_smax), 1e-30f) * (GAL ? 3.1f : 1.f) * 8.f;
-            int e2;
-            frexpf(m, &e2);
-            qs = (T)ldexpf(1.f, 32 - e2);
-            iq = (T)ldexpf(1.f, e2 - 32);
-        }
-    }
 
     // ---- the row table of the source rows into shared memory, when it fits: every node of a
     //      row reads that row's entry, and a shared-memory load is shorter than an L1 hit
@@ -998,12 +950,97 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         const float4 *from = reinterpret_cast<const float4 *>(A.row + ja);
         float4 *to = reinterpret_cast<float4 *>(rowc);
         for (int k = tid; k < kVec * (jb - ja + 1); k += blockDim.x) to[k] = __ldg(from + k);
-        __syncthreads();
     }
     const RowEntry<T> *srow = rowc - ja;   // srow[j]: row j (rows_cached only)
 
+    // ---- FP32: fixed-point scale of the window from max|s| over the rows the walk reads, taken
+    //      from the per-tile maxima the previous step (or vp_set_f) recorded for the state.
+    //      The truncated Thomas solve keeps |w| <= 3 max|s| (forward gain 1/(beta - 1/6) <= 2.2,
+    //      back substitution 1/(1 - c') <= 1.37); a cell sums the B3 taps of the nodes pushed near
+    //      it, about one for an area-preserving flow: 8 times that bound fits in int32.
+    T qs = T(1), iq = T(1);
+    if (sizeof(T) == 4) {
+        // every warp for itself: no exchange between warps
+        unsigned mx = 0u;   // bits of a non-negative float: ordered as the float
+        const unsigned *map = reinterpret_cast<const unsigned *>(A.smax_in);
+        if (jb >= ja) {
+            const int r0 = GAL ? max(0, ja - kHalo) : ja, r1 = GAL ? min(np - 1, jb + kHalo) : jb;
+            const int c0 = imod(ia, nx), c1 = c0 + min(ib - ia + 1, nx) - 1;
+            // tile columns the source columns c0 .. c1 (wrapped) lie in
+            const int t0 = c0 / A.tx, nt = (c1 < nx ? c1 / A.tx : A.ntx + (c1 - nx) / A.tx) - t0 + 1;
+            const int q0 = r0 / A.tp, nq = r1 / A.tp - q0 + 1;
+            for (int k = lane; k < nt * nq; k += 32) {
+                const int q = k / nt;
+                int tc = t0 + k - q * nt;
+                if (tc >= A.ntx) tc -= A.ntx;
+                mx = max(mx, map[(q0 + q) * A.ntx + tc]);
+            }
+        }
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (!(__uint_as_float(mx) <= 3.0e38f)) {
+            qs = T(0);   // a non-finite state, reported when it was written: its deposit is dropped
+            iq = T(0);
+        } else {
+            // the scale is a power of two, so that iq = 1 / qs is exact (a rounded iq scales the
+            // tile's weights by 1 +- 6e-8, a gain that repeats over the steps while the tile's
+            // maximum stays put): qs = 2^(32 - e) with m = f 2^e, f in [0.5, 1), i.e. qs m in
+            // [2^31, 2^32): a cell reaches 2^31 only at 4 to 8 times the largest weight (16 to 32
+            // times with the Thomas gain bound), against about one for an area-preserving flow
+            // (a floor of 1e-28 keeps qs finite where the state is zero)
+            const float m = fmaxf(__uint_as_float(mx), 1e-28f) * (GAL ? 3.1f : 1.f) * 8.f;
+            int e2;
+            frexpf(m, &e2);
+            qs = (T)ldexpf(1.f, 32 - e2);
+            iq = (T)ldexpf(1.f, e2 - 32);
+        }
+    }
+    __syncthreads();   // the zeroed window, the row table, the pivots
+
     // ---- walk the source columns
-    if (jb >= ja) {
+    if constexpr (sizeof(T) == 4) {
+        // FP32: items of (pair of adjacent columns, segment of rows). The first column of every pair is
+        // even where the mesh allows, so that a pair's source values are one 8-byte load
+        const int wmax = nx, ia2 = (nx & 1) == 0 && ib - ia + 2 <= nx ? ia - (ia & 1) : ia;
+        const int wsrc = jb >= ja ? min(ib - ia2 + 1, wmax) : 0;
+        const int npair = (wsrc + 1) >> 1;
+        const int rows = jb - ja + 1, nseg = min(A.nseg, max(1, rows / kMinSegRows)), len = (rows + nseg - 1) / nseg;
+        Walk32 K;
+        K.src = A.src;
+        K.nx = nx;
+        K.np = np;
+        K.row = A.row;
+        K.rowc = smem_addr(rowc) - (unsigned)ja * (unsigned)sizeof(RowEntry<float>);
+        K.piv = piv32;
+        K.W = &s_win;
+        K.win = smem_addr(win);
+        K.ws4 = W.ws * 4;
+        K.lim = W.WH * W.ws * 4;
+        K.WW = W.WW;
+        K.WP0 = W.WP0;
+        K.edge = (P0 == 0 ? 1 : 0) | (P0 + TPe == np ? 2 : 0);
+        // kept in registers: rebuilt from the arguments at every use they cost 20 of 200 instructions a row
+        K.ws4 = opaque(K.ws4);
+        K.lim = opaque(K.lim);
+        K.edge = opaque(K.edge);
+        const unsigned gc = smem_addr(gcol) + 8u * tid, gs = 8u * blockDim.x;
+        // a warp's lanes share their segment (a warp over two segments runs both, one after the other)
+        const int nwp = (npair + 31) >> 5;
+        for (int wi = warp; wi < nwp * nseg; wi += nwarps) {
+            const int sg = wi / nwp, q = (wi - sg * nwp) * 32 + lane, ic = ia2 + 2 * q;
+            const int r_lo = ja + sg * len, r_hi = min(jb, r_lo + len - 1);
+            if (q >= npair || r_lo > r_hi) continue;
+            const int imA = imod(ic, nx), imB = imA + 1 < nx ? imA + 1 : 0;
+            // a last pair of one column: its second column takes the weight 0
+            const bool two = ic + 1 - ia2 < wsrc;
+            const f2_t q2 = f2_pack(qs, two ? qs : 0.f);
+            if (rows_cached)
+                walk_pair<BASIS, GAL, UTERM, true>(K, A.col[imA], A.col[imB], imA, imB, ic - W.WX0, r_lo, r_hi, q2,
+                                                   (float)al, (float)be, (float)g.KU, (float)g.KV, gc, gs, lost);
+            else
+                walk_pair<BASIS, GAL, UTERM, false>(K, A.col[imA], A.col[imB], imA, imB, ic - W.WX0, r_lo, r_hi, q2,
+                                                    (float)al, (float)be, (float)g.KU, (float)g.KV, gc, gs, lost);
+        }
+    } else if (jb >= ja) {
         int wsrc = ib - ia + 1;
         if (wsrc > nx) wsrc = nx;
         const T alT = (T)al, beT = (T)be, KU = (T)g.KU, KV = (T)g.KV;
@@ -1053,7 +1090,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
 #pragma unroll 1
                         for (int r = c_lo; r <= c_hi; ++r) {
                             int m, n;
-                            node_taps<T, BASIS, UTERM, true>(cc, srow[r], colrel, r - W.WP0,
+                            node_taps<T, BASIS, UTERM>(cc, srow[r], colrel, r - W.WP0,
                                                              gc[(r - c_lo) * nth] * qs, m, n, wx, wy);
                             ring_add<T, N, 1>(win, W, rg, m, n, wx, wy, lost);
                         }
@@ -1061,7 +1098,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
 #pragma unroll 1
                         for (int r = c_lo; r <= c_hi; ++r) {
                             int m, n;
-                            node_taps<T, BASIS, UTERM, false>(cc, A.row[r], colrel, r - W.WP0,
+                            node_taps<T, BASIS, UTERM>(cc, A.row[r], colrel, r - W.WP0,
                                                               gc[(r - c_lo) * nth] * qs, m, n, wx, wy);
                             ring_add<T, N, 1>(win, W, rg, m, n, wx, wy, lost);
                         }
@@ -1130,7 +1167,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
                         for (int r = c_hi; r >= c_lo; --r, --rp) {
                             uv = gc[(r - c_lo) * nth] - cp_inf * uv;
                             int m, n;
-                            node_taps<T, BASIS, UTERM, true>(cc, *rp, colrel, r - W.WP0, uv * qs, m, n, wx, wy);
+                            node_taps<T, BASIS, UTERM>(cc, *rp, colrel, r - W.WP0, uv * qs, m, n, wx, wy);
                             ring_add<T, N, -1>(win, W, rg, m, n, wx, wy, lost);
                         }
                     } else if (c_lo > kPivots) {
@@ -1139,7 +1176,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
                         for (int r = c_hi; r >= c_lo; --r, --rp) {
                             uv = gc[(r - c_lo) * nth] - cp_inf * uv;
                             int m, n;
-                            node_taps<T, BASIS, UTERM, false>(cc, *rp, colrel, r - W.WP0, uv * qs, m, n, wx, wy);
+                            node_taps<T, BASIS, UTERM>(cc, *rp, colrel, r - W.WP0, uv * qs, m, n, wx, wy);
                             ring_add<T, N, -1>(win, W, rg, m, n, wx, wy, lost);
                         }
                     } else {
@@ -1147,7 +1184,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
                         for (int r = c_hi; r >= c_lo; --r, --rp) {
                             uv = gc[(r - c_lo) * nth] - piv_cp[min(r, kPivots)] * uv;
                             int m, n;
-                            node_taps<T, BASIS, UTERM, false>(cc, *rp, colrel, r - W.WP0, uv * qs, m, n, wx, wy);
+                            node_taps<T, BASIS, UTERM>(cc, *rp, colrel, r - W.WP0, uv * qs, m, n, wx, wy);
                             ring_add<T, N, -1>(win, W, rg, m, n, wx, wy, lost);
                         }
                     }
@@ -1188,17 +1225,24 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         // row pass solves Lambda_x, records max|s'| per tile and checks the outputs
         store_window_rows<T, false>(win, W, A.dst, nx, P0, X0, TXe, TPe, G, Gp, iq, warp, nwarps, lane, om, bad);
     } else if (GAL) {
-        const int L = full ? nx : TXe + 2 * D;
-        const bool f32 = sizeof(T) == 4;
-        const T sh = f32 ? (T)A.piv[kPivXsFused] : T(-6) * T(-0.26794919243112270647);
-        const T sl = f32 ? (T)A.piv[kPivXsFused + 1] : T(0);
-        if (L <= 256)
-            gal_rows<T, 8>(win, W, A.dst, L, full, D, G, Gp, TXe, TPe, P0, X0, nx, want_part, warp,
-                           nwarps, lane, bad, gcol, GRows<T>::value * blockDim.x, sh, sl, iq, om);
-        else
-            gal_rows<T, kXBig>(win, W, A.dst, L, full, D, G, Gp, TXe, TPe, P0, X0, nx, want_part,
-                               warp, nwarps, lane, bad, gcol, GRows<T>::value * blockDim.x, sh, sl, iq,
-                               om);
+        if constexpr (sizeof(T) == 4) {
+            const float sh = (float)A.piv[kPivXsFused], sl = (float)A.piv[kPivXsFused + 1];
+            if ((full ? nx : A.tx) + 2 * kHalo <= 256)
+                solve_rows_f32<8>(win, W, A.dst, full, G, Gp, TXe, TPe, P0, X0, nx, want_part, warp, nwarps, lane, sh,
+                                  sl, iq, om, bad);
+            else
+                solve_rows_f32<kXBig32>(win, W, A.dst, full, G, Gp, TXe, TPe, P0, X0, nx, want_part, warp, nwarps, lane,
+                                        sh, sl, iq, om, bad);
+        } else {
+            const int L = full ? nx : TXe + 2 * D;
+            const T sh = T(-6) * T(-0.26794919243112270647), sl = T(0);
+            if (L <= 256)
+                gal_rows<T, 8>(win, W, A.dst, L, full, D, G, Gp, TXe, TPe, P0, X0, nx, want_part, warp, nwarps, lane,
+                               bad, gcol, GRows<T>::value * blockDim.x, sh, sl, iq, om);
+            else
+                gal_rows<T, kXBig>(win, W, A.dst, L, full, D, G, Gp, TXe, TPe, P0, X0, nx, want_part, warp, nwarps,
+                                   lane, bad, gcol, GRows<T>::value * blockDim.x, sh, sl, iq, om);
+        }
     } else {
         // no solve: the deposit is the new state (its max|w| sets the next step's window scale)
         store_window_rows<T, true>(win, W, A.dst, nx, P0, X0, TXe, TPe, G, Gp, iq, warp, nwarps, lane, om, bad);
@@ -1209,7 +1253,11 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         // those of s')
         __syncthreads();
         const bool sums_of_s = GAL && !A.xpass;
-        for (int c = tid; c < TXe; c += blockDim.x) {
+        // columns go to kSumWarps virtual warps whatever the block size, so that a simulation's sums are
+        // formed in the same order alone and in a batch
+        for (int vw = warp; vw < kSumWarps; vw += nwarps) {
+        pw = pc = ps = 0.0;
+        for (int c = vw * 32 + lane; c < TXe; c += 32 * kSumWarps) {
             // four interleaved compensated sums (rows rr = q mod 4), added in a fixed order at the
             // end: four independent chains of shared-memory loads and error-free steps instead of one
             DSum<T> acc[4];
@@ -1240,33 +1288,41 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         }
         pc *= A.bunch_x;
         ps *= A.bunch_x;
+        for (int o = 16; o > 0; o >>= 1) {
+            pw += __shfl_down_sync(0xffffffffu, pw, o);
+            pc += __shfl_down_sync(0xffffffffu, pc, o);
+            ps += __shfl_down_sync(0xffffffffu, ps, o);
+        }
+        if (lane == 0) {
+            s_part[0][vw] = pw;
+            s_part[1][vw] = pc;
+            s_part[2][vw] = ps;
+        }
+        }
     }
     if (bad) atomicOr(A.err, ERRF_NONFINITE);
 
     // ---- per-tile reductions in a fixed order (FP64 work only where there is weight to sum)
     // FP32: record max|s'| of the tile for the next step's window scale
     if (sizeof(T) == 4 && om > 0.f) atomicMax(&s_omax, __float_as_int(om));
-    const bool reduce = __syncthreads_or(lost != 0.0 || want_part);
+    const bool any_lost = __syncthreads_or(lost != 0.0);
     if (sizeof(T) == 4 && tid == 0) A.smax_out[tile] = __int_as_float(s_omax);
-    if (!reduce) return;
-    // lost weight back to weight units: iq = 1 / qs exactly (a power of two; 0 for a dropped deposit)
-    double vals[4] = {lost * (double)iq, pw, pc, ps};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        double v = vals[q];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) s_r4[q][warp] = v;
+    if (want_part && tid < 3) {
+        double t = 0.0;
+        for (int w = 0; w < kSumWarps; ++w) t += s_part[tid][w];
+        A.tile_part[3 * tile + tid] = t;
+        __threadfence();   // visible before thread 0 takes the step's ticket
     }
-    __syncthreads();
-    if (tid == 0) {
-        double t[4] = {0, 0, 0, 0};
-        for (int q = 0; q < 4; ++q)
-            for (int w = 0; w < nwarps; ++w) t[q] += s_r4[q][w];
-        A.tile_lost[tile] += t[0];
-        if (want_part) {
-            A.tile_part[3 * tile + 0] = t[1];
-            A.tile_part[3 * tile + 1] = t[2];
-            A.tile_part[3 * tile + 2] = t[3];
+    if (any_lost) {
+        // back to weight units: iq = 1 / qs exactly (a power of two; 0 for a dropped deposit)
+        double v = lost * (double)iq;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) s_lost[warp] = v;
+        __syncthreads();
+        if (tid == 0) {
+            double t = 0.0;
+            for (int w = 0; w < nwarps; ++w) t += s_lost[w];
+            A.tile_lost[tile] += t;
         }
     }
 }
@@ -1302,7 +1358,8 @@ __device__ __forceinline__ void finish_step(const FusedArgs<T> &A, unsigned char
 }
 
 template <typename T, int BASIS, bool GAL, bool UTERM, int MINB>
-__global__ void __launch_bounds__(MINB == 1 ? kFusedMaxThreads : kFusedThreads2, MINB)
+__global__ void __launch_bounds__(sizeof(T) == 4 ? kFusedThreads32 : (MINB == 1 ? kFusedMaxThreads : kFusedThreads2),
+                                  sizeof(T) == 4 ? 512 / kFusedThreads32 : MINB)
     step_fused_kernel(const FusedArgs<T> A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1316,8 +1373,8 @@ __global__ void __launch_bounds__(MINB == 1 ? kFusedMaxThreads : kFusedThreads2,
 // once the instance has taken its steps (left[k] == 0). One CTA per item rather than a persistent
 // loop over an atomic counter: inside a loop the compiler kept the arguments of every item live
 // and spilled 400 bytes per thread; one item per CTA spills 60.
-template <typename T, int BASIS, bool GAL, bool UTERM, int MINB>
-__global__ void __launch_bounds__(MINB == 1 ? kFusedMaxThreads : kFusedThreads2, MINB)
+template <typename T, int BASIS, bool GAL, bool UTERM>
+__global__ void __launch_bounds__(kFusedThreads32, 512 / kFusedThreads32)
     step_fused_batch_kernel(const FusedArgs<T> *__restrict__ args, const int *__restrict__ parity,
                             const int *__restrict__ left, const int2 *__restrict__ items, int nitems)
 {
@@ -1353,8 +1410,8 @@ int fused_rowcache_rows(int precision, size_t base_bytes, int ctas)
         if (cudaDeviceGetAttribute(&v, cudaDevAttrReservedSharedMemoryPerBlock, dev) == cudaSuccess) reserved = v;
         cudaFuncAttributes fa;
         const void *k = precision == VP_FP64
-                            ? reinterpret_cast<const void *>(step_fused_batch_kernel<double, VP_BASIS_CUBIC_BSPLINE, true, true, 2>)
-                            : reinterpret_cast<const void *>(step_fused_batch_kernel<float, VP_BASIS_CUBIC_BSPLINE, true, true, 2>);
+                            ? reinterpret_cast<const void *>(step_fused_kernel<double, VP_BASIS_CUBIC_BSPLINE, true, true, 2>)
+                            : reinterpret_cast<const void *>(step_fused_batch_kernel<float, VP_BASIS_CUBIC_BSPLINE, true, true>);
         if (cudaFuncGetAttributes(&fa, k) == cudaSuccess) stat = fa.sharedSizeBytes + 256;
         cudaGetLastError();
     }
@@ -1378,8 +1435,9 @@ cudaError_t launch_step_fused(const FusedArgs<T> &a, int threads, cudaStream_t s
     const bool uterm = a.g.kind == VP_PUSH_FEL_DKD;
 #define VP_LAUNCH_FUSED(B, GL, UT)                                                            \
     do {                                                                                      \
-        auto k = threads > kFusedThreads2 ? step_fused_kernel<T, B, GL, UT, 1>                 \
-                                          : step_fused_kernel<T, B, GL, UT, 2>;                \
+        auto k = step_fused_kernel<T, B, GL, UT, 2>;                                          \
+        if constexpr (sizeof(T) == 8)                                                         \
+            if (threads > kFusedThreads2) k = step_fused_kernel<T, B, GL, UT, 1>;              \
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
                                              (int)smem);                                      \
         if (e != cudaSuccess) return e;                                                       \
@@ -1475,8 +1533,7 @@ cudaError_t launch_step_fused_batch(const FusedArgs<T> *args, const int *parity,
     const bool gal = basis == VP_BASIS_CUBIC_BSPLINE && projection == VP_PROJ_GALERKIN;
 #define VP_LAUNCH_BATCH(B, GL)                                                                \
     do {                                                                                      \
-        auto k = threads > kFusedThreads2 ? step_fused_batch_kernel<T, B, GL, true, 1>         \
-                                          : step_fused_batch_kernel<T, B, GL, true, 2>;        \
+        auto k = step_fused_batch_kernel<T, B, GL, true>;                                     \
         if (grid <= 0) /* set-up call: shared-memory attribute only (not capturable) */       \
             return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
                                         (int)smem);                                           \
@@ -1494,17 +1551,9 @@ cudaError_t launch_step_fused_batch(const FusedArgs<T> *args, const int *parity,
 int fused_batch_blocks_per_sm(int basis, int projection, size_t smem, int threads)
 {
     const bool gal = basis == VP_BASIS_CUBIC_BSPLINE && projection == VP_PROJ_GALERKIN;
-    const void *k = nullptr;
-    const bool one = threads > kFusedThreads2;
-    if (basis == VP_BASIS_TENT)
-        k = one ? (const void *)step_fused_batch_kernel<float, VP_BASIS_TENT, false, true, 1>
-                : (const void *)step_fused_batch_kernel<float, VP_BASIS_TENT, false, true, 2>;
-    else if (!gal)
-        k = one ? (const void *)step_fused_batch_kernel<float, VP_BASIS_CUBIC_BSPLINE, false, true, 1>
-                : (const void *)step_fused_batch_kernel<float, VP_BASIS_CUBIC_BSPLINE, false, true, 2>;
-    else
-        k = one ? (const void *)step_fused_batch_kernel<float, VP_BASIS_CUBIC_BSPLINE, true, true, 1>
-                : (const void *)step_fused_batch_kernel<float, VP_BASIS_CUBIC_BSPLINE, true, true, 2>;
+    const void *k = (const void *)step_fused_batch_kernel<float, VP_BASIS_CUBIC_BSPLINE, true, true>;
+    if (basis == VP_BASIS_TENT) k = (const void *)step_fused_batch_kernel<float, VP_BASIS_TENT, false, true>;
+    else if (!gal) k = (const void *)step_fused_batch_kernel<float, VP_BASIS_CUBIC_BSPLINE, false, true>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -1940,9 +1989,6 @@ template cudaError_t launch_xsolve_rows<double>(const double *, double *, int, i
 template cudaError_t launch_step_fused_batch<float>(const FusedArgs<float> *, const int *, const int *,
                                                     const int2 *, int, int, int, size_t, int, int,
                                                     cudaStream_t);
-template cudaError_t launch_step_fused_batch<double>(const FusedArgs<double> *, const int *, const int *,
-                                                     const int2 *, int, int, int, size_t, int, int,
-                                                     cudaStream_t);
 template size_t fused_smem_bytes<float>(int, int, int, int);
 template size_t fused_smem_bytes<double>(int, int, int, int);
 template cudaError_t launch_step_fused<float>(const FusedArgs<float> &, int, cudaStream_t);
