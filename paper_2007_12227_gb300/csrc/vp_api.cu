@@ -23,7 +23,7 @@ namespace {
 constexpr size_t kAlign = 256;
 constexpr int kDefaultHist = 4096;
 constexpr size_t kMaxSmem = 220 * 1024;
-constexpr int kMoutLen = 32;
+constexpr int kMoutLen = kMoutState + ST_NSTATE + 1;   // moments, step state, error flags
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
@@ -626,11 +626,9 @@ vp_status reset_state(vp_sim *s, const void *w)
     return VP_OK;
 }
 
-vp_status check_flags(vp_sim *s)
+// the status the error flags last read (host_err) stand for
+vp_status flag_status(vp_sim *s)
 {
-    VP_CUDA(s, cudaMemcpyAsync(&s->host_err, s->ws + s->P.L.err, sizeof(unsigned),
-                               cudaMemcpyDeviceToHost, s->stream));
-    VP_CUDA(s, cudaStreamSynchronize(s->stream));
     if (s->host_err & ERRF_NONFINITE)
         return fail(s->msg, VP_ERR_NONFINITE, "a step produced a non-finite weight");
     if (s->host_err & ERRF_TIMEOUT)
@@ -638,6 +636,13 @@ vp_status check_flags(vp_sim *s)
     return VP_OK;
 }
 
+vp_status check_flags(vp_sim *s)
+{
+    VP_CUDA(s, cudaMemcpyAsync(&s->host_err, s->ws + s->P.L.err, sizeof(unsigned),
+                               cudaMemcpyDeviceToHost, s->stream));
+    VP_CUDA(s, cudaStreamSynchronize(s->stream));
+    return flag_status(s);
+}
 }  // namespace
 
 extern "C" {
@@ -875,6 +880,23 @@ static void *host_device_ptr(const void *p, size_t align)
     return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
 }
 
+// The caller's device buffer, when a kernel on the sim's device can take it in place of a copy: memory of the
+// current device (a copy also takes memory of a peer without access to it), aligned to its elements, outside
+// the sim's own workspace (vp_state_device hands out the buffer that vp_set_f writes).
+static void *own_device_ptr(const vp_sim *s, const void *p, size_t align)
+{
+    if ((uintptr_t)p % align) return nullptr;
+    const char *q = static_cast<const char *>(p), *end = q + (size_t)s->P.g.nx * s->P.g.np * align;
+    if (q < s->ws + s->P.L.total && end > s->ws) return nullptr;
+    cudaPointerAttributes at;
+    int dev = -1;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == dev ? const_cast<void *>(p) : nullptr;
+}
+
 enum class Xfer { host, device, host_async };
 
 static vp_status set_f_common(vp_sim *s, const void *src, int32_t dtype, size_t n, Xfer mode)
@@ -891,10 +913,12 @@ static vp_status set_f_common(vp_sim *s, const void *src, int32_t dtype, size_t 
     const size_t szs = P.precision == VP_FP64 ? 8 : 4;
     if (async && dtype != P.precision)
         return fail(s->msg, VP_ERR_ARG, "set_f_async: the weights must have the simulation's dtype");
-    // pinned host weights and the state s = Lambda_p w: Lambda_p reads them in place (the
+    // pinned host or device weights and the state s = Lambda_p w: Lambda_p reads them in place (the
     // asynchronous call copies them with the copy engine instead, which overlaps other streams'
     // transfers in the opposite direction)
-    void *hdev = (!device && !async && dtype == P.precision && P.state_s) ? host_device_ptr(src, szs) : nullptr;
+    void *hdev = nullptr;
+    if (!async && dtype == P.precision && P.state_s)
+        hdev = device ? own_device_ptr(s, src, szs) : host_device_ptr(src, szs);
     if (hdev) {
         dst = hdev;
     } else if (dtype == P.precision) {
@@ -925,25 +949,27 @@ static vp_status set_f_common(vp_sim *s, const void *src, int32_t dtype, size_t 
     s->f_set = true;
     vp_status st = reset_state(s, dst);
     if (st != VP_OK) return st;
+    const bool maxima = P.kernel == VP_KERNEL_FUSED && P.precision == VP_FP32;
     if (P.state_s) {
         if (P.precision == VP_FP64)
             VP_CUDA(s, launch_lambda_p_mul<double>(static_cast<const double *>(dst),
-                                                   static_cast<double *>(s->f(0)), P.g.nx, P.g.np,
-                                                   s->stream));
+                                                   static_cast<double *>(s->f(0)), P.g.nx, P.g.np, nullptr,
+                                                   0, 0, 0, 0, s->ptr<unsigned>(P.L.err), s->stream));
         else
             VP_CUDA(s, launch_lambda_p_mul<float>(static_cast<const float *>(dst),
                                                   static_cast<float *>(s->f(0)), P.g.nx, P.g.np,
-                                                  s->stream));
+                                                  s->ptr<float>(P.L.smax), P.tx, P.tp, P.ntx, P.ntp,
+                                                  s->ptr<unsigned>(P.L.err), s->stream));
+    } else if (maxima) {
+        VP_CUDA(s, launch_tile_max(static_cast<const float *>(s->f(0)), s->ptr<float>(P.L.smax), P.g.nx,
+                                   P.g.np, P.tx, P.tp, P.ntx, P.ntp, s->ptr<unsigned>(P.L.err),
+                                   s->stream));
     }
     if (P.fel && !P.rk4 && P.g.sigma2 != 0.0) {
         const vp_status sc = P.precision == VP_FP64 ? fel_space_charge<double>(s, s->f(0))
                                                     : fel_space_charge<float>(s, s->f(0));
         if (sc != VP_OK) return sc;
     }
-    if (P.kernel == VP_KERNEL_FUSED && P.precision == VP_FP32)
-        VP_CUDA(s, launch_tile_max(static_cast<const float *>(s->f(0)), s->ptr<float>(P.L.smax), P.g.nx,
-                                   P.g.np, P.tx, P.tp, P.ntx, P.ntp, s->ptr<unsigned>(P.L.err),
-                                   s->stream));
     // the caller owns the host buffer again once vp_set_f returns; the asynchronous form leaves it
     // to the caller's vp_sync
     if (mode == Xfer::host) VP_CUDA(s, cudaStreamSynchronize(s->stream));
@@ -1023,16 +1049,18 @@ static vp_status get_f_common(vp_sim *s, void *dstp, int32_t dtype, size_t n, Xf
         return fail(s->msg, VP_ERR_ARG, "get_f_async: the weights must have the simulation's dtype");
     const void *src = nullptr;
     const size_t szs = P.precision == VP_FP64 ? 8 : 4;
-    // a pinned host buffer and the state s = Lambda_p w: the p solve writes the weights in place
+    // a pinned host or a device buffer and the state s = Lambda_p w: the p solve writes the weights in place
     // (the asynchronous call solves into device memory and copies with the copy engine)
-    void *hdev = (!device && !async && dtype == P.precision && P.state_s) ? host_device_ptr(dstp, szs) : nullptr;
+    void *hdev = nullptr;
+    if (!async && dtype == P.precision && P.state_s)
+        hdev = device ? own_device_ptr(s, dstp, szs) : host_device_ptr(dstp, szs);
     {
         vp_status st = P.precision == VP_FP64 ? weights_of_state<double>(s, &src, hdev)
                                               : weights_of_state<float>(s, &src, hdev);
         if (st != VP_OK) return st;
     }
     if (hdev) {
-        // the p solve above wrote the weights into the host buffer
+        // the p solve above wrote the weights into the caller's buffer
     } else if (dtype == P.precision) {
         VP_CUDA(s, cudaMemcpyAsync(dstp, src, N * szs,
                                    device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
@@ -1096,13 +1124,15 @@ vp_status vp_moments(vp_sim *s, vp_moments_t *out)
     else
         VP_CUDA(s, launch_moments<float>(static_cast<const float *>(w), P.g,
                                          s->ptr<double2>(P.L.csx), mpart, P.nmblk, s->stream));
+    // the sums, then the step state and the error flags beside them: one copy to the host
     VP_CUDA(s, launch_moments_finalize(mpart, P.nmblk, s->ptr<double>(P.L.lost), P.nlost, mout,
-                                       s->stream));
+                                       s->ptr<double>(P.L.state), s->ptr<unsigned>(P.L.err), s->stream));
     VP_CUDA(s, cudaMemcpyAsync(s->host_mout, mout, kMoutLen * sizeof(double), cudaMemcpyDeviceToHost,
                                s->stream));
-    VP_CUDA(s, cudaMemcpyAsync(s->host_state, s->ws + P.L.state, sizeof(s->host_state),
-                               cudaMemcpyDeviceToHost, s->stream));
-    vp_status st = check_flags(s);
+    VP_CUDA(s, cudaStreamSynchronize(s->stream));
+    memcpy(s->host_state, s->host_mout + kMoutState, sizeof(s->host_state));
+    s->host_err = (unsigned)s->host_mout[kMoutState + ST_NSTATE];
+    vp_status st = flag_status(s);
     const double *m = s->host_mout;
     const double hh = P.g.hx * P.g.hp;
     const double S = m[0];

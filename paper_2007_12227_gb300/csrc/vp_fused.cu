@@ -1458,70 +1458,123 @@ cudaError_t launch_step_fused(const FusedArgs<T> &a, int threads, cudaStream_t s
 }
 
 // s = Lambda_p w along columns (tridiag(1/6, 2/3, 1/6), zero beyond the open edges). Each thread
-// walks one column through a chunk of kMulRows rows, so every input row is read once (plus a halo
+// walks one column through a chunk of rows, so every input row is read once (plus a halo
 // row at either end of the chunk): w may be host memory the device reads in place.
-constexpr int kMulRows = 64;
+// MAX: also max|s| over each tx x tp tile into the zeroed map[][ntx] (infinity, and the error flag, where a
+// value is not finite), which as a pass of its own read the state once more (0.137 ms for 8192 x 8192).
 constexpr int kMulCols = 256;
 
-template <typename T>
-__global__ void __launch_bounds__(kMulCols)
-    lambda_p_mul_kernel(const T *__restrict__ w, T *__restrict__ s, int nx, int np)
+// m (bits of a non-negative float) of the columns of one warp into their tiles of one tile row
+__device__ __forceinline__ void max_to_map(unsigned m, int col, int nx, int tx, unsigned *map_row)
 {
-    const int col = blockIdx.x * kMulCols + threadIdx.x;
-    if (col >= nx) return;
-    const int j0 = blockIdx.y * kMulRows, j1 = min(j0 + kMulRows, np);
-    T lo = j0 > 0 ? w[(size_t)(j0 - 1) * nx + col] : T(0);
-    T c = w[(size_t)j0 * nx + col];
-#pragma unroll 8
-    for (int j = j0; j < j1; ++j) {
-        const T hi = j + 1 < np ? w[(size_t)(j + 1) * nx + col] : T(0);
-        s[(size_t)j * nx + col] = (lo + hi) * (T(1) / T(6)) + c * (T(2) / T(3));
-        lo = c;
-        c = hi;
+    const int t0 = __shfl_sync(0xffffffffu, col, 0) / tx, t = min(col, nx - 1) / tx;
+    if (__all_sync(0xffffffffu, t == t0)) {
+        m = __reduce_max_sync(0xffffffffu, m);
+        if ((threadIdx.x & 31) == 0 && m != 0u) atomicMax(map_row + t0, m);
+    } else if (m != 0u) {
+        atomicMax(map_row + t, m);
     }
 }
 
-// max|s| per tile (one CTA per tile); a non-finite value sets the error flag
-__global__ void tile_max_kernel(const float *__restrict__ s, float *__restrict__ map, int nx, int np,
-                                int tx, int tp, int ntx, unsigned *err)
+template <typename T, bool MAX>
+__global__ void __launch_bounds__(kMulCols)
+    lambda_p_mul_kernel(const T *__restrict__ w, T *__restrict__ s, int nx, int np, int rows, unsigned *map, int tx,
+                        int tp, int ntx, unsigned *err)
 {
-    __shared__ int s_m, s_bad;
-    if (threadIdx.x == 0) {
-        s_m = 0;
-        s_bad = 0;
+    const int col = blockIdx.x * kMulCols + threadIdx.x;
+    if (!MAX && col >= nx) return;
+    const bool in = col < nx;
+    const int j0 = blockIdx.y * rows, j1 = min(j0 + rows, np);
+    T lo = in && j0 > 0 ? w[(size_t)(j0 - 1) * nx + col] : T(0);
+    T c = in ? w[(size_t)j0 * nx + col] : T(0);
+    for (int ja = j0; ja < j1;) {   // rows of one tile row at a time
+        const int jb = MAX ? min(j1, (ja / tp + 1) * tp) : j1;
+        float m = 0.f, chk = 0.f;
+#pragma unroll 8
+        for (int j = ja; j < jb; ++j) {
+            const T hi = in && j + 1 < np ? w[(size_t)(j + 1) * nx + col] : T(0);
+            const T v = (lo + hi) * (T(1) / T(6)) + c * (T(2) / T(3));
+            if (in) s[(size_t)j * nx + col] = v;
+            if (MAX) {
+                m = fmaxf(m, fabsf((float)v));
+                chk = fmaf((float)v, 0.f, chk);   // 0, or NaN once a value is not finite
+            }
+            lo = c;
+            c = hi;
+        }
+        if (MAX) {
+            if (chk != 0.f) {
+                m = __int_as_float(0x7f800000);
+                atomicOr(err, ERRF_NONFINITE);
+            }
+            max_to_map(__float_as_uint(m), col, nx, tx, map + (size_t)(ja / tp) * ntx);
+        }
+        ja = jb;
     }
-    __syncthreads();
-    const int X0 = (blockIdx.x % ntx) * tx, P0 = (blockIdx.x / ntx) * tp;
-    const int TX = min(tx, nx - X0), TP = min(tp, np - P0);
-    float m = 0.f, chk = 0.f;
-    for (int k = threadIdx.x; k < TX * TP; k += blockDim.x) {
-        const int r = k / TX, c = k - r * TX;
-        const float v = s[(size_t)(P0 + r) * nx + X0 + c];
-        m = fmaxf(m, fabsf(v));
-        chk = fmaf(v, 0.f, chk);
+}
+
+// max|s| per tile of a state that is there already (no solve, so nothing else passes over it), into the zeroed
+// map: a warp takes 32 columns of a chunk of rows, as above
+__global__ void __launch_bounds__(kMulCols)
+    tile_max_kernel(const float *__restrict__ s, unsigned *map, int nx, int np, int rows, int tx, int tp, int ntx,
+                    unsigned *err)
+{
+    const int col = blockIdx.x * kMulCols + threadIdx.x;
+    const bool in = col < nx;
+    const int j0 = blockIdx.y * rows, j1 = min(j0 + rows, np);
+    for (int ja = j0; ja < j1;) {
+        const int jb = min(j1, (ja / tp + 1) * tp);
+        float m = 0.f, chk = 0.f;
+#pragma unroll 16
+        for (int j = ja; j < jb; ++j) {
+            const float v = in ? s[(size_t)j * nx + col] : 0.f;
+            m = fmaxf(m, fabsf(v));
+            chk = fmaf(v, 0.f, chk);
+        }
+        if (chk != 0.f) {
+            m = __int_as_float(0x7f800000);
+            atomicOr(err, ERRF_NONFINITE);
+        }
+        max_to_map(__float_as_uint(m), col, nx, tx, map + (size_t)(ja / tp) * ntx);
+        ja = jb;
     }
-    if (m > 0.f) atomicMax(&s_m, __float_as_int(m));
-    if (chk != 0.f) s_bad = 1;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        map[blockIdx.x] = s_bad ? __int_as_float(0x7f800000) : __int_as_float(s_m);
-        if (s_bad) atomicOr(err, ERRF_NONFINITE);
-    }
+}
+
+// rows per block of the two kernels above: 64, or 16 where 64 would leave most SMs without a block
+static int column_rows(int nx, int np)
+{
+    const long blocks = (long)((nx + kMulCols - 1) / kMulCols) * ((np + 63) / 64);
+    int rows = blocks < 152 * 4 ? 16 : 64;
+    while ((np + rows - 1) / rows > 65535) rows *= 2;
+    return rows;
 }
 
 cudaError_t launch_tile_max(const float *s, float *map, int nx, int np, int tx, int tp, int ntx,
                             int ntp, unsigned *err, cudaStream_t st)
 {
-    tile_max_kernel<<<ntx * ntp, 256, 0, st>>>(s, map, nx, np, tx, tp, ntx, err);
+    const int rows = column_rows(nx, np);
+    cudaError_t e = cudaMemsetAsync(map, 0, (size_t)ntx * ntp * sizeof(float), st);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((nx + kMulCols - 1) / kMulCols, (np + rows - 1) / rows);
+    tile_max_kernel<<<grid, kMulCols, 0, st>>>(s, reinterpret_cast<unsigned *>(map), nx, np, rows, tx, tp, ntx, err);
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_lambda_p_mul(const T *w, T *s, int nx, int np, cudaStream_t st)
+cudaError_t launch_lambda_p_mul(const T *w, T *s, int nx, int np, float *map, int tx, int tp, int ntx, int ntp,
+                                unsigned *err, cudaStream_t st)
 {
-    const dim3 grid((nx + kMulCols - 1) / kMulCols, (np + kMulRows - 1) / kMulRows);
-    if (grid.y > 65535u) return cudaErrorInvalidConfiguration;
-    lambda_p_mul_kernel<T><<<grid, kMulCols, 0, st>>>(w, s, nx, np);
+    const int rows = column_rows(nx, np);
+    const dim3 grid((nx + kMulCols - 1) / kMulCols, (np + rows - 1) / rows);
+    if ((np + 63) / 64 > 65535) return cudaErrorInvalidConfiguration;
+    if (map) {
+        cudaError_t e = cudaMemsetAsync(map, 0, (size_t)ntx * ntp * sizeof(float), st);
+        if (e != cudaSuccess) return e;
+        lambda_p_mul_kernel<T, true><<<grid, kMulCols, 0, st>>>(w, s, nx, np, rows, reinterpret_cast<unsigned *>(map), tx,
+                                                                tp, ntx, err);
+    } else {
+        lambda_p_mul_kernel<T, false><<<grid, kMulCols, 0, st>>>(w, s, nx, np, rows, nullptr, 1, 1, 1, err);
+    }
     return cudaGetLastError();
 }
 
@@ -1993,7 +2046,9 @@ template size_t fused_smem_bytes<float>(int, int, int, int);
 template size_t fused_smem_bytes<double>(int, int, int, int);
 template cudaError_t launch_step_fused<float>(const FusedArgs<float> &, int, cudaStream_t);
 template cudaError_t launch_step_fused<double>(const FusedArgs<double> &, int, cudaStream_t);
-template cudaError_t launch_lambda_p_mul<float>(const float *, float *, int, int, cudaStream_t);
-template cudaError_t launch_lambda_p_mul<double>(const double *, double *, int, int, cudaStream_t);
+template cudaError_t launch_lambda_p_mul<float>(const float *, float *, int, int, float *, int, int, int, int,
+                                                unsigned *, cudaStream_t);
+template cudaError_t launch_lambda_p_mul<double>(const double *, double *, int, int, float *, int, int, int, int,
+                                                 unsigned *, cudaStream_t);
 
 }  // namespace vp

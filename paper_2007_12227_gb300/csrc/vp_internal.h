@@ -248,8 +248,10 @@ cudaError_t launch_xsolve_rows(const T *r, T *out, int nx, int np, const double 
                                int ntx, float *smax_out, unsigned *err, int grid, cudaStream_t s);
 constexpr int kFusedMaxRow = 512; // longest window row one warp solves
 constexpr int kFusedMaxTileP = 256; // tallest tile of the fused kernel
+// s = Lambda_p w; map (may be NULL): max|s| per tile as launch_tile_max gives it
 template <typename T>
-cudaError_t launch_lambda_p_mul(const T *w, T *s, int nx, int np, cudaStream_t st);
+cudaError_t launch_lambda_p_mul(const T *w, T *s, int nx, int np, float *map, int tx, int tp, int ntx, int ntp,
+                                unsigned *err, cudaStream_t st);
 // max|s| of an FP32 state over each tile x tile_p tile into map[ntp][ntx]; non-finite -> err
 cudaError_t launch_tile_max(const float *s, float *map, int nx, int np, int tx, int tp, int ntx,
                             int ntp, unsigned *err, cudaStream_t st);
@@ -307,8 +309,11 @@ template <typename T>
 cudaError_t launch_moments(const T *w, const Geometry &g, const double2 *csx, double *part,
                            int nblocks, cudaStream_t s);
 int moment_blocks(int nx, int np);
+// out: the kNumMoments sums and the lost weight, the step state from kMoutState on, then the error flags
+constexpr int kMoutState = 16;
 cudaError_t launch_moments_finalize(const double *part, int nblocks, const double *lost,
-                                    int nlost, double *out, cudaStream_t s);
+                                    int nlost, double *out, const double *state, const unsigned *err,
+                                    cudaStream_t s);
 
 template <typename Tin, typename Tout>
 cudaError_t launch_convert(const Tin *in, Tout *out, size_t n, cudaStream_t s);

@@ -174,52 +174,157 @@ __global__ void count_step_kernel(double *state, double dt)
     state[ST_TAU] = st * dt;
 }
 
-// w ln w in FP64, for FP32 weights too (the entropy is an FP64 reduction)
-template <typename T>
-__device__ __forceinline__ double wlogw(T w)
+// Moments. Bound by the FP64 pipe (2 operations per clock and SM on this GPU), not by memory: 62 FP64
+// operations a node took 0.45 ms for 2048 x 2048 (0.28 ms now, the final sums 12 us against 153 in one thread
+// each). A warp therefore walks 32 columns through a chunk of rows and
+// keeps per column only the sums over p (w, w p, w p^2: everything else of a node's moments is a factor of its
+// column), the entropy, and the negative and the trapped weight: about a dozen.
+//
+// w ln w of FP32 weights: with w = 2^e m and c the centre of m's 512th of [1, 2), u = m / c - 1 (|u| < 2^-10),
+// ln w = (e ln 2 + ln c) + ln(1 + u), the series of ln(1 + u) cut after u^5 / 5 (the next term is below 2^-62). 1 / c
+// is rounded, so ln c in the table is minus the log of that rounded value: u carries one rounding, of order 2^-53.
+constexpr int kLnBits = 9, kLnTab = 1 << kLnBits;
+struct LnTable {
+    double2 c[kLnTab];   // rounded 1 / c, and -ln of it
+    double e[256];       // (e - 127) ln 2
+};
+
+__device__ __forceinline__ void ln_table(LnTable &t)
 {
-    const double d = (double)w;
-    return d * log(d);
+    for (int k = threadIdx.x; k < kLnTab; k += blockDim.x) {
+        const double ic = 1.0 / (1.0 + (k + 0.5) / kLnTab);
+        t.c[k] = make_double2(ic, -log(ic));
+    }
+    for (int k = threadIdx.x; k < 256; k += blockDim.x) t.e[k] = (k - 127) * 0.693147180559945309417;
+}
+
+// conversion by integer operations where it can be (a conversion instruction runs at the FP64 rate)
+__device__ __forceinline__ double wide_of(float w)
+{
+    const unsigned b = __float_as_uint(w), e = (b >> 23) & 255u;
+    if (e == 0u || e == 255u) return (double)w;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double wide_of(double w) { return w; }
+
+__device__ __forceinline__ double ln_of(float w, const LnTable &t)
+{
+    const unsigned b = __float_as_uint(w);
+    const int e = (int)(b >> 23);
+    if (e == 0 || e == 255) return log((double)w);   // denormal or not finite
+    const unsigned man = b & 0x7fffffu;
+    const double m = __hiloint2double((int)(0x3ff00000u | (man >> 3)), (int)(man << 29));
+    const double2 q = t.c[man >> (23 - kLnBits)];
+    const double u = fma(m, q.x, -1.0);
+    double s = fma(u, 0.2, -0.25);
+    s = fma(u, s, 1.0 / 3.0);
+    s = fma(u, s, -0.5);
+    s = fma(u, s, 1.0);
+    return fma(u, s, t.e[e] + q.y);
+}
+__device__ __forceinline__ double ln_of(double w, const LnTable &) { return log(w); }
+
+// rows of a warp's chunk and the chunks of a column (the same on the host and in the kernel)
+__host__ __device__ __forceinline__ int moment_rows(int nx, int np)
+{
+    // about 8 warps on each of the 8 blocks of an SM; at least 8 rows, so that the column factors are spread
+    const long long strips = (nx + 31) / 32, want = 152LL * 8 * 8;
+    const long long chunks = want / strips < 1 ? 1 : want / strips;
+    const long long rows = (np + chunks - 1) / chunks;
+    return rows < 8 ? 8 : (int)rows;
 }
 
 template <typename T>
-__global__ void moments_kernel(const T *__restrict__ w, Geometry g, const double2 *__restrict__ csx,
-                               double *part)
+__global__ void __launch_bounds__(kRedThreads)
+    moments_kernel(const T *__restrict__ w, Geometry g, const double2 *__restrict__ csx, double *part)
 {
     __shared__ double s_red[kNumMoments][kRedThreads / 32];
+    __shared__ LnTable s_ln;
+    if (sizeof(T) == 4) ln_table(s_ln);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
     double acc[kNumMoments];
 #pragma unroll
     for (int q = 0; q < kNumMoments; ++q) acc[q] = 0.0;
-    const size_t n = (size_t)g.nx * g.np;
     const double hsep = fabs(g.v_sign);
     const bool pend = (g.kind == VP_PUSH_LEAPFROG_KDK && g.potential == VP_POT_PENDULUM);
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const T wt = w[idx];
-        if (wt == T(0)) continue;
-        const int j = (int)(idx / g.nx), i = (int)(idx - (size_t)j * g.nx);
-        const double x = g.x0 + i * g.hx, p = g.p0 + j * g.hp;
-        const double ww = (double)wt;
+    const int rows = moment_rows(g.nx, g.np);
+    const long long strips = (g.nx + 31) / 32, chunks = (g.np + rows - 1) / rows, ntask = strips * chunks;
+    for (long long task = (long long)blockIdx.x * (kRedThreads / 32) + wy; task < ntask;
+         task += (long long)gridDim.x * (kRedThreads / 32)) {
+        const int i0 = (int)(task % strips) * 32 + lane, i = min(i0, g.nx - 1);
+        const bool in = i0 < g.nx;
+        const int r0 = (int)(task / strips) * rows, r1 = min(r0 + rows, g.np);
+        const double x = g.x0 + i * g.hx;
         const double2 cs = csx[i];
         double V = 0.0;
         if (g.potential == VP_POT_PENDULUM) V = -g.v_sign * cs.x;
         else if (g.potential == VP_POT_HARMONIC) V = 0.5 * g.omega * g.omega * x * x;
-        const double H = 0.5 * p * p + V;
-        acc[0] += ww;
-        acc[1] += ww * x;
-        acc[2] += ww * p;
-        acc[3] += ww * x * x;
-        acc[4] += ww * p * p;
-        acc[5] += ww * x * p;
-        acc[6] += ww * H;
-        if (pend && H < hsep) acc[7] += ww;
-        if (wt > T(0)) acc[8] -= wlogw(wt);
-        else acc[9] += ww;
-        acc[10] += ww * cs.x;
-        acc[11] += ww * cs.y;
-        acc[12] = fmax(acc[12], fabs(ww));
+        // sums over the column's chunk. s0 collects the weight of the present side of the separatrix, t0 that of
+        // the other: they change places where the column crosses it
+        double s0 = 0.0, t0 = 0.0, s1 = 0.0, s2 = 0.0, ent = 0.0, neg = 0.0, mx = 0.0;
+        bool inside = false;
+        float mxf = 0.f;
+        const T *src = w + (size_t)r0 * g.nx + i;
+        constexpr int F = 8;   // loads in flight
+        T v[F];
+        auto load = [&](int r) -> T { return in && r < r1 ? __ldg(src + (size_t)(r - r0) * g.nx) : T(0); };
+#pragma unroll
+        for (int k = 0; k < F; ++k) v[k] = load(r0 + k);
+        const float vf = (float)(V - hsep);
+        double p_of = 0.0;   // lane l: the momentum of row rb + l, for 32 rows at a time
+        float pf_of = 0.f;
+        for (int rb = r0; rb < r1; rb += F) {
+            const int ph = (rb - r0) & 31;
+            if (ph == 0) {
+                p_of = g.p0 + (rb + lane) * g.hp;
+                pf_of = (float)p_of;
+            }
+#pragma unroll
+            for (int k = 0; k < F; ++k) {
+                const int r = rb + k;
+                const T wt = v[k];
+                v[k] = load(r + F);
+                const double p = __shfl_sync(0xffffffffu, p_of, ph + k);
+                const float pf = __shfl_sync(0xffffffffu, pf_of, ph + k);
+                if (wt == T(0)) continue;   // also rows past the chunk and columns past the mesh
+                const double ww = wide_of(wt);
+                if (pend) {
+                    // H < hsep as FP64 gives it; FP32 decides where it is not close
+                    const float hf = 0.5f * pf * pf + vf;
+                    const bool now = fabsf(hf) > 1e-5f * (pf * pf + 4.f * (float)hsep) ? hf < 0.f : 0.5 * p * p + V < hsep;
+                    if (now != inside) {
+                        const double o = s0;
+                        s0 = t0;
+                        t0 = o;
+                        inside = now;
+                    }
+                }
+                s0 += ww;
+                const double wp = ww * p;
+                s1 += wp;
+                s2 = fma(wp, p, s2);
+                if (wt > T(0)) ent = fma(-ww, ln_of(wt, s_ln), ent);
+                else neg += ww;
+                if (sizeof(T) == 4) mxf = fmaxf(mxf, fabsf((float)wt));
+                else mx = fmax(mx, fabs(ww));
+            }
+        }
+        const double sw = s0 + t0;
+        acc[0] += sw;
+        acc[1] = fma(sw, x, acc[1]);
+        acc[2] += s1;
+        acc[3] = fma(sw * x, x, acc[3]);
+        acc[4] += s2;
+        acc[5] = fma(s1, x, acc[5]);
+        acc[6] += fma(sw, V, 0.5 * s2);
+        acc[7] += inside ? s0 : (pend ? t0 : 0.0);
+        acc[8] += ent;
+        acc[9] += neg;
+        acc[10] = fma(sw, cs.x, acc[10]);
+        acc[11] = fma(sw, cs.y, acc[11]);
+        acc[12] = fmax(acc[12], sizeof(T) == 4 ? (double)mxf : mx);
     }
-    const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
 #pragma unroll
     for (int q = 0; q < kNumMoments; ++q) {
         double v = acc[q];
@@ -234,25 +339,29 @@ __global__ void moments_kernel(const T *__restrict__ w, Geometry g, const double
         const int q = threadIdx.x;
         double t = 0.0;
         for (int k = 0; k < kRedThreads / 32; ++k) t = (q == 12) ? fmax(t, s_red[q][k]) : t + s_red[q][k];
-        part[(size_t)blockIdx.x * kNumMoments + q] = t;
+        part[(size_t)q * gridDim.x + blockIdx.x] = t;
     }
 }
 
-__global__ void moments_finalize_kernel(const double *__restrict__ part, int nblocks,
-                                        const double *__restrict__ lost, int nlost, double *out)
+// one warp per sum (a strided pass, then a tree: a fixed order), the last one the lost weight and the copies
+__global__ void __launch_bounds__(32 * (kNumMoments + 1))
+    moments_finalize_kernel(const double *__restrict__ part, int nblocks, const double *__restrict__ lost, int nlost,
+                            double *out, const double *__restrict__ state, const unsigned *__restrict__ err)
 {
-    const int q = threadIdx.x;
-    if (q < kNumMoments) {
-        double t = 0.0;
-        for (int b = 0; b < nblocks; ++b) {
-            const double v = part[(size_t)b * kNumMoments + q];
-            t = (q == 12) ? fmax(t, v) : t + v;
-        }
-        out[q] = t;
-    } else if (q == kNumMoments) {
-        double t = 0.0;
-        for (int b = 0; b < nlost; ++b) t += lost[b];
-        out[q] = t;
+    const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double *v = q < kNumMoments ? part + (size_t)q * nblocks : lost;
+    const int n = q < kNumMoments ? nblocks : nlost;
+    double t = 0.0;
+#pragma unroll 8
+    for (int b = lane; b < n; b += 32) t = (q == 12) ? fmax(t, v[b]) : t + v[b];
+    for (int o = 16; o > 0; o >>= 1) {
+        const double u = __shfl_down_sync(0xffffffffu, t, o);
+        t = (q == 12) ? fmax(t, u) : t + u;
+    }
+    if (lane == 0) out[q] = t;
+    if (q == kNumMoments) {
+        for (int k = lane; k < ST_NSTATE; k += 32) out[kMoutState + k] = state[k];
+        if (lane == 0) out[kMoutState + ST_NSTATE] = (double)*err;
     }
 }
 
@@ -320,10 +429,10 @@ cudaError_t launch_count_step(double *state, double dt, cudaStream_t s)
 
 int moment_blocks(int nx, int np)
 {
-    const size_t n = (size_t)nx * np;
-    size_t b = (n + kRedThreads - 1) / kRedThreads;
-    if (b > 152 * 8) b = 152 * 8;
-    return (int)b;
+    const int rows = moment_rows(nx, np);
+    const long long tasks = (long long)((nx + 31) / 32) * ((np + rows - 1) / rows);
+    const long long b = (tasks + kRedThreads / 32 - 1) / (kRedThreads / 32);
+    return (int)(b < 152 * 8 ? b : 152 * 8);
 }
 
 template <typename T>
@@ -335,9 +444,9 @@ cudaError_t launch_moments(const T *w, const Geometry &g, const double2 *csx, do
 }
 
 cudaError_t launch_moments_finalize(const double *part, int nblocks, const double *lost, int nlost,
-                                    double *out, cudaStream_t s)
+                                    double *out, const double *state, const unsigned *err, cudaStream_t s)
 {
-    moments_finalize_kernel<<<1, 32, 0, s>>>(part, nblocks, lost, nlost, out);
+    moments_finalize_kernel<<<1, 32 * (kNumMoments + 1), 0, s>>>(part, nblocks, lost, nlost, out, state, err);
     return cudaGetLastError();
 }
 
