@@ -23,6 +23,8 @@ namespace {
 constexpr size_t kAlign = 256;
 constexpr int kDefaultHist = 4096;
 constexpr size_t kMaxSmem = 220 * 1024;
+constexpr int kAutoXpassRow64 = 288;
+constexpr int kSlots = 2 * 152;   // CTAs of the step kernel the chip holds (two per SM)
 constexpr int kMoutLen = kMoutState + ST_NSTATE + 1;   // moments, step state, error flags
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -43,8 +45,9 @@ struct Plan {
     int rowcache;   // fused kernel: row-table rows a tile may cache in shared memory
     int nseg;       // fused kernel, FP32: row segments per pair of source columns
     bool full_row, state_s;
-    // Galerkin one-pass plan with a separate x pass: tiles without x halo store the deposit into
-    // tmp, and a row pass solves Lambda_x along whole rows into the state buffer
+    // Galerkin one-pass plan with a separate x pass: tiles without x halo store the deposit into tmp (x_in_place:
+    // into the state buffer), and a row pass solves Lambda_x along whole rows into the state buffer
+    bool x_in_place;
     bool xpass;
     int xgrid;   // CTAs of the row pass (persistent)
     bool rk4;   // FEL with the RK4 integrator: the scatter kernel and stage reductions
@@ -162,6 +165,16 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
         P->xpass = true;
         kernel = VP_KERNEL_FUSED;
     }
+    // FP64 Galerkin by the planner's choice: rows longer than two windows take the separate x pass. An in-tile
+    // solve needs 28 columns on both sides of a tile (1.5 times the tile's own columns at 112), all of them
+    // through the FP64 pipe; batches, which take the one-pass form only, hold FP32
+    const bool auto_x = kernel == VP_KERNEL_AUTO && opts->precision == VP_FP64 && P->galerkin && !P->rk4 &&
+                        !wide_rotation && grid->nx >= kAutoXpassRow64;
+    if (auto_x) {
+        int xt = 0, xper = 0;
+        xrow_shape(opts->precision, grid->nx, &xt, &xper);
+        if (xt > 0 && xrow_smem_bytes(opts->precision, grid->nx, 0) <= kMaxSmem) P->xpass = true;
+    }
     if (P->rk4 || basis == VP_BASIS_SEPTIC_BSPLINE) {
         // the RK4 end point is not of the tabulated displacement form, and the 8-tap septic
         // deposit has no one-pass form here: global-atomic deposit
@@ -183,13 +196,13 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
         const int halo = P->galerkin && !P->xpass ? fused_halo(opts->precision) : 0;
         const int R = basis == VP_BASIS_TENT ? 1 : 2;
         const int G = P->G, Gp = P->Gp;
-        ftx = opts->tile_x ? opts->tile_x : (opts->precision == VP_FP64 ? 128 : (halo ? 208 : 240));
+        ftx = opts->tile_x ? opts->tile_x : (opts->precision == VP_FP64 ? 112 : (halo ? 208 : 240));
         ftp = opts->tile_p ? opts->tile_p : 64;
         bool full = false;
         // whole-period tiles when the mesh is little wider than a windowed tile; by default only
         // while the tile's source columns fit the two-CTA thread count (a default plan of more
         // threads runs one CTA per SM, and in a batch it would set that for every item)
-        const bool full_fits = (grid->nx + 2 * R + 8 + 31) / 32 * 32 <= kFusedThreads2;
+        const bool full_fits = (grid->nx + 2 * R + 8 + 31) / 32 * 32 <= 320;
         if (!P->xpass && grid->nx <= kFusedMaxRow && grid->nx < ftx + 2 * halo + 2 * G + 64 &&
             (full_fits || opts->tile_x != 0 || grid->nx <= ftx + 2 * halo + 2 * G)) {
             full = true;
@@ -197,29 +210,81 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
         }
         if (!full && ftx + 2 * halo > kFusedMaxRow) ftx = kFusedMaxRow - 2 * halo;
         ftp = std::min(std::min(ftp, grid->np), kFusedMaxTileP);
+        const bool pick64 = sz == 8 && !full && opts->tile_x == 0;
+        if (pick64) {
+            // FP64: the tile's time is the FP64 pipe's, so the shape with the least walked work per slot: lanes in
+            // whole warps times the rows walked (the tile's, the B3 reach, and what the p solve of its row segments
+            // adds), times the waves. (1024 x 1024: 56 x 64, exactly one wave, 240 us; 112 x 36 285; 128 x 16 with
+            // an in-tile x solve 485.)
+            double best = 1e300;
+            int bw = ftx, bh = ftp;
+            for (int lanes = 64; lanes <= 256; lanes += 32) {
+                const int w = lanes - 2 * halo - 2 * R - 4, wsz = (w + 2 * halo + 2 * G + 31) / 32 * 32;
+                if (w < 24 || w + 2 * halo + 2 * G >= grid->nx) continue;
+                for (int h = 8; h <= 64; h += 4) {
+                    const int hh = opts->tile_p ? ftp : std::min(h, grid->np);
+                    const int seg = std::max(1, std::min(kFusedThreads / lanes, hh / 8));
+                    if (fused_smem_bytes<double>(wsz, hh + 2 * Gp, lanes * seg) > (size_t)112 * 1024) continue;
+                    const double tiles = (double)((grid->nx + w - 1) / w) * ((grid->np + hh - 1) / hh);
+                    const double cost = ceil(tiles / kSlots) * lanes * (hh + 7 + (P->galerkin ? 4 * seg : 0));
+                    if (cost < best) {
+                        best = cost;
+                        bw = w;
+                        bh = hh;
+                    }
+                }
+            }
+            ftx = bw;
+            ftp = bh;
+        }
         const int WW = full ? grid->nx + 2 * G : ftx + 2 * halo + 2 * G;
         // row stride a multiple of 32 words: the rows start 16-byte aligned, and lanes that
         // deposit into adjacent columns of two neighbouring rows hit distinct banks
         const int ws = (WW + 31) / 32 * 32;
-        const int wsrc = (full ? grid->nx : ftx + 2 * halo) + 2 * R + 8;
-        // two CTAs per SM (up to 320 threads) unless the tile is wide: then one CTA of up
-        // to 576 threads per SM
-        const bool wide = (wsrc + 31) / 32 * 32 > kFusedThreads2;
-        int threads = std::min(wide ? kFusedMaxThreads : kFusedThreads2, (wsrc + 31) / 32 * 32);
-        int nseg = 1;
-        if (sz == 4) {
-            // a thread walks a pair of columns through a segment of the tile's rows: as many segments as
-            // the block's threads serve in one round
-            const int lanes = (wsrc / 2 + 1 + 31) / 32 * 32;
-            nseg = std::max(1, std::min(kFusedThreads32 / lanes, ftp / 8));
-            threads = std::min(kFusedThreads32, lanes * nseg);
-        }
+        const int wsrc = (full ? grid->nx : ftx + 2 * halo) + 2 * R + (pick64 ? 4 : 8);
+        // two CTAs per SM unless the tile is wide
+        const bool wide = wsrc > 320;   // one CTA per SM
         const size_t cap = wide ? (size_t)200 * 1024 : (size_t)112 * 1024;
+        if (opts->tile_p == 0 && !pick64) {
+            const int ntx = (grid->nx + ftx - 1) / ftx;
+            auto tiles = [&](int h) { return (long)ntx * ((grid->np + h - 1) / h); };
+            if (tiles(ftp) <= kSlots) {
+                // a mesh that does not fill the chip with such tiles: as low as gives every slot one (a tile's time
+                // is a fixed part of some 30 rows' worth plus its rows: 357 x 300 FP32 takes 37 us a step with 64
+                // rows, 22.8 with 24, 18.7 with 16; but in a batch, where other simulations fill the chip, low tiles
+                // only add the fixed part: 40 mixed ones take 132, 117 and 140 us)
+                const int least = opts->precision == VP_FP64 ? 4 : 24;   // FP64 here: whole-period tiles, not in batches
+                const int per_col = std::max(1, kSlots / ntx), h = (grid->np + per_col - 1) / per_col;
+                ftp = std::min(ftp, std::max(least, (h + 3) / 4 * 4));
+            } else {
+                // a last wave of less than 0.4 of the slots costs nearly a whole one: lower tiles fill it (2048 x 2048
+                // FP32: 64 rows, 1.05 waves, 59.8 us a step; 48 rows, 1.41 waves, 49.5 us)
+                for (int h = ftp; h >= 40 && h <= 64; h -= 4) {
+                    const double waves = (double)tiles(h) / kSlots, last = waves - floor(waves);
+                    if (waves > 8.0 || last == 0.0 || last >= 0.4) {
+                        ftp = h;
+                        break;
+                    }
+                }
+            }
+        }
+        // a thread walks a pair (FP64: one) of source columns through a segment of the tile's rows: as many
+        // segments as the block's threads serve in one round
+        const int lanes = ((sz == 4 ? wsrc / 2 + 1 : wsrc) + 31) / 32 * 32;
+        int threads = 0, nseg = 1;
+        auto split_rows = [&](int tp_) {
+            nseg = std::max(1, std::min(kFusedThreads / lanes, tp_ / 8));
+            threads = std::min(kFusedThreads, lanes * nseg);
+        };
+        split_rows(ftp);
         auto smem_of = [&](int tp_) {
             return sz == 8 ? fused_smem_bytes<double>(ws, tp_ + 2 * Gp, threads)
                            : fused_smem_bytes<float>(ws, tp_ + 2 * Gp, threads);
         };
-        while (smem_of(ftp) > cap && ftp > 8) ftp /= 2;
+        while (smem_of(ftp) > cap && ftp > 8) {
+            ftp /= 2;
+            split_rows(ftp);
+        }
         const size_t smem = smem_of(ftp);
         const bool ok = !wide_rotation && smem <= kMaxSmem && (full || WW < grid->nx) && ftx >= 1;
         if (ok) {
@@ -290,9 +355,12 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
     L.f0 = take(N * sz);
     L.f1 = take(N * sz);
     // a third mesh-sized buffer only where a step needs one: the deposit between the two launches of
-    // the separate-x-pass plan, the x-solve output of the separate-filter path. The one-pass plan
-    // reads its weights out through the idle ping-pong buffer instead
-    L.tmp = take(((P->galerkin && (kernel != VP_KERNEL_FUSED || P->xpass)) || P->septic_gal) ? N * sz : 0);
+    // the separate-x-pass plan when asked for, the x-solve output of the separate-filter path. The one-pass plan
+    // reads its weights out through the idle ping-pong buffer; the planner's own choice of a separate x pass
+    // needs no more memory than the one-pass plan (its rows are solved in place)
+    P->x_in_place = P->xpass && opts->kernel != VP_KERNEL_FUSED_XPASS;
+    L.tmp = take(((P->galerkin && (kernel != VP_KERNEL_FUSED || (P->xpass && !P->x_in_place))) || P->septic_gal)
+                     ? N * sz : 0);
     L.col = take(grid->nx * colsz);
     L.row = take(grid->np * rowsz);
     L.rowb = take(grid->np * sizeof(RowBound));
@@ -508,8 +576,8 @@ vp_status do_steps(vp_sim *s, int n, cudaEvent_t *ev = nullptr)
         void *src = s->f(s->cur), *dst = s->f(1 - s->cur);
         StepArgs<T> a = step_args<T>(s, src, dst);
         if (P.kernel == VP_KERNEL_FUSED) {
-            // separate x pass: the tiles store the deposit into tmp, the row pass solves it into dst
-            void *tile_dst = P.xpass ? static_cast<void *>(s->ptr<T>(P.L.tmp)) : dst;
+            // separate x pass: the tiles store the deposit into tmp (or dst), the row pass solves it into dst
+            void *tile_dst = P.xpass && !P.x_in_place ? static_cast<void *>(s->ptr<T>(P.L.tmp)) : dst;
             VP_CUDA(s, launch_step_fused<T>(fused_args<T>(s, src, tile_dst), P.threads, s->stream));
         } else if (P.kernel == VP_KERNEL_TILED) {
             VP_CUDA(s, launch_step_tiled<T>(a, s->stream));
@@ -532,7 +600,8 @@ vp_status do_steps(vp_sim *s, int n, cudaEvent_t *ev = nullptr)
             if (P.xpass) {
                 float *m0 = s->ptr<float>(P.L.smax);
                 float *mout = P.precision == VP_FP32 ? (src == s->f(0) ? m0 + (size_t)P.ntx * P.ntp : m0) : nullptr;
-                VP_CUDA(s, launch_xsolve_rows<T>(s->ptr<T>(P.L.tmp), static_cast<T *>(dst), P.g.nx, P.g.np,
+                VP_CUDA(s, launch_xsolve_rows<T>(P.x_in_place ? static_cast<T *>(dst) : s->ptr<T>(P.L.tmp),
+                                                 static_cast<T *>(dst), P.g.nx, P.g.np,
                                                  s->ptr<double>(P.L.piv), P.tx, P.tp, P.ntx, mout, err,
                                                  P.xgrid, s->stream));
                 if (e) {

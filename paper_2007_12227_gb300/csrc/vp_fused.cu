@@ -35,6 +35,7 @@
 #include "vp_internal.h"
 #include "vp_sum.cuh"
 #include "vp_walk.cuh"
+#include "vp_walk64.cuh"
 
 namespace vp {
 namespace {
@@ -45,49 +46,16 @@ template <typename T>
 struct Halo {
     static constexpr int value = sizeof(T) == 4 ? 16 : 28;
 };
+constexpr int kMaxGroups = 16;      // groups of 64 source columns whose rows are bounded on their own
 constexpr int kSumWarps = 8;        // virtual warps of the per-tile FEL column sums
 constexpr int kMinSegRows = 8;      // shortest row segment of the FP32 walk (each restarts its rings)
-constexpr int kC = 16;              // rows per chunk of the p solve (multiple of 4)
-// elements of the per-thread column buffer: one chunk of rows, or the look-ahead above the top row;
-// FP32 threads walk two columns
+// elements of the per-thread column buffer: one chunk of rows; FP32 threads walk two columns
 template <typename T>
 struct GRows {
-    static constexpr int value = sizeof(T) == 4 ? 2 * kC32 : (kC > Halo<T>::value ? kC : Halo<T>::value);
+    static constexpr int value = sizeof(T) == 4 ? 2 * kC32 : kC64;
 };
 constexpr int kXBig = kFusedMaxRow / 32;   // elements per lane for rows up to kFusedMaxRow
 constexpr int kXBig32 = 20;                // FP32: whole-period rows of kFusedMaxRow with the halo on both sides
-
-template <typename T, int BASIS>
-struct FTaps;
-
-template <typename T>
-struct FTaps<T, VP_BASIS_TENT> {
-    static constexpr int N = 2;
-    static constexpr int LO = 0;
-    __device__ __forceinline__ static void weights(T t, T *w)
-    {
-        w[0] = T(1) - t;
-        w[1] = t;
-    }
-};
-
-template <typename T>
-struct FTaps<T, VP_BASIS_CUBIC_BSPLINE> {
-    static constexpr int N = 4;
-    static constexpr int LO = -1;
-    // cubic B-spline at offsets 1+t, t, 1-t, 2-t
-    __device__ __forceinline__ static void weights(T t, T *w)
-    {
-        const T s = T(1) - t;
-        const T t2 = t * t, s2 = s * s;
-        const T t3 = t2 * t, s3 = s2 * s;
-        const T sixth = T(1) / T(6), two3 = T(2) / T(3);
-        w[0] = s3 * sixth;
-        w[3] = t3 * sixth;
-        w[1] = two3 - t2 + T(0.5) * t3;
-        w[2] = ((T(1) - w[0]) - w[3]) - w[1];
-    }
-};
 
 __device__ __forceinline__ int imod(int a, int n)
 {
@@ -139,7 +107,6 @@ __device__ void sin_range32(float lo, float hi, float &smin, float &smax)
 // native integer shared-memory atomics (a float atomicAdd on shared memory is a
 // compare-and-swap loop) and the sums do not depend on the order of the additions: the
 // FP32 step is bit-reproducible. FP64: doubles.
-__device__ __forceinline__ void wadd(double *p, double v) { atomicAdd(p, v); }
 // raw cell value (in the tile's scaled units)
 __device__ __forceinline__ double wraw(const float *p) { return (double)*reinterpret_cast<const int *>(p); }
 __device__ __forceinline__ double wraw(const double *p) { return *p; }
@@ -155,15 +122,6 @@ __device__ __forceinline__ void wfold(float *d, const float *s)
 }
 __device__ __forceinline__ void wfold(double *d, const double *s) { *d += *s; }
 
-template <typename T, int N>
-struct Ring {
-    T acc[N][N];  // [slot][column]
-    int mref;     // window column of tap a = 0
-    int nb;       // window row of tap b = 0 of the last node
-    bool col_ok;  // all N columns inside the window
-    bool live;
-};
-
 struct WinGeom {
     int WW, WH, ws;      // window width, height, row stride (elements)
     int WX0, WP0;        // grid column (unwrapped) and row of window cell (0, 0)
@@ -171,195 +129,6 @@ struct WinGeom {
     int np, nx, G;
     bool full;           // the tile spans the whole period
 };
-
-// One cell outside the fast window range: wrap (whole-period tiles), add, or count
-// as lost (rows beyond the open momentum edge, own columns). Returns the lost weight.
-template <typename T>
-__device__ __noinline__ double flush_cell_slow(T *win, const WinGeom W, T v, int c, int row)
-{
-    if (W.full && (c < 0 || c >= W.WW)) c = W.G + imod(c - W.G, W.nx);
-    const int grow = row + W.WP0;
-    const bool outside = grow < 0 || grow >= W.np;
-    if (c >= 0 && c < W.WW) {
-        if (row >= 0 && row < W.WH) {
-            wadd(win + row * W.ws + c, v);
-            return 0.0;
-        }
-        if (outside && (W.full || (c >= W.own_c0 && c < W.own_c1))) return (double)v;
-    }
-    return 0.0;
-}
-
-template <typename T>
-__device__ __forceinline__ void flush_cell(T *win, const WinGeom &W, T v, int c, int row, double &lost)
-{
-    if (row >= 0 && row < W.WH && c >= 0 && c < W.WW) wadd(win + row * W.ws + c, v);
-    else lost += flush_cell_slow<T>(win, W, v, c, row);
-}
-
-template <typename T, int N>
-__device__ __forceinline__ void flush_row(T *win, const WinGeom &W, const T *acc, int mref,
-                                          bool col_ok, int row, double &lost)
-{
-    if (row >= 0 && row < W.WH && col_ok) {
-        T *p = win + row * W.ws + mref;
-#pragma unroll
-        for (int a = 0; a < N; ++a) wadd(p + a, acc[a]);
-    } else {
-#pragma unroll
-        for (int a = 0; a < N; ++a) lost += flush_cell_slow<T>(win, W, acc[a], mref + a, row);
-    }
-}
-
-// Add one node (weights wx, wy; base window column m, row n). acc[b] always holds
-// window row nb + b. DIR = +1: base rows ascend between consecutive nodes (the
-// bottom row leaves); DIR = -1: they descend (the top row leaves). The row shift
-// is folded into the accumulation: acc[b] = acc[b +/- 1] + wy[b] wx.
-template <typename T, int N, int DIR>
-__device__ __forceinline__ void ring_add(T *win, const WinGeom &W, Ring<T, N> &rg, int m, int n,
-                                         const T *wx, const T *wy, double &lost)
-{
-    {
-        // common case: one row leaves the ring, nothing else changes. Each lane decides for
-        // itself (a warp vote here measured slower: lanes that fail diverge only briefly)
-        const int rl = DIR > 0 ? rg.nb : rg.nb + N - 1;
-        const bool fast = rg.live && n == rg.nb + DIR && m == rg.mref && rg.col_ok &&
-                          (unsigned)rl < (unsigned)W.WH;
-        if (fast) {
-            T *p = win + rl * W.ws + rg.mref;
-            if (DIR > 0) {
-#pragma unroll
-                for (int a = 0; a < N; ++a) wadd(p + a, rg.acc[0][a]);
-#pragma unroll
-                for (int b = 0; b < N - 1; ++b)
-#pragma unroll
-                    for (int a = 0; a < N; ++a) rg.acc[b][a] = rg.acc[b + 1][a] + wy[b] * wx[a];
-#pragma unroll
-                for (int a = 0; a < N; ++a) rg.acc[N - 1][a] = wy[N - 1] * wx[a];
-            } else {
-#pragma unroll
-                for (int a = 0; a < N; ++a) wadd(p + a, rg.acc[N - 1][a]);
-#pragma unroll
-                for (int b = N - 1; b > 0; --b)
-#pragma unroll
-                    for (int a = 0; a < N; ++a) rg.acc[b][a] = rg.acc[b - 1][a] + wy[b] * wx[a];
-#pragma unroll
-                for (int a = 0; a < N; ++a) rg.acc[0][a] = wy[0] * wx[a];
-            }
-            rg.nb = n;
-            return;
-        }
-    }
-    const bool step_ok = rg.live && n == rg.nb + DIR;
-    if (step_ok && (m == rg.mref + 1 || m == rg.mref - 1)) {
-        // the base column moved by one: flush the column that leaves, shift the rest
-        if (m > rg.mref) {
-#pragma unroll
-            for (int b = 0; b < N; ++b) {
-                flush_cell<T>(win, W, rg.acc[b][0], rg.mref, rg.nb + b, lost);
-#pragma unroll
-                for (int a = 0; a < N - 1; ++a) rg.acc[b][a] = rg.acc[b][a + 1];
-                rg.acc[b][N - 1] = T(0);
-            }
-        } else {
-#pragma unroll
-            for (int b = 0; b < N; ++b) {
-                flush_cell<T>(win, W, rg.acc[b][N - 1], rg.mref + N - 1, rg.nb + b, lost);
-#pragma unroll
-                for (int a = N - 1; a > 0; --a) rg.acc[b][a] = rg.acc[b][a - 1];
-                rg.acc[b][0] = T(0);
-            }
-        }
-        rg.mref = m;
-        rg.col_ok = (unsigned)m <= (unsigned)(W.WW - N);   // overflow-safe for any m
-    }
-    if (step_ok && m == rg.mref) {
-        if (DIR > 0) {
-            flush_row<T, N>(win, W, rg.acc[0], rg.mref, rg.col_ok, rg.nb, lost);
-#pragma unroll
-            for (int b = 0; b < N - 1; ++b)
-#pragma unroll
-                for (int a = 0; a < N; ++a) rg.acc[b][a] = rg.acc[b + 1][a] + wy[b] * wx[a];
-#pragma unroll
-            for (int a = 0; a < N; ++a) rg.acc[N - 1][a] = wy[N - 1] * wx[a];
-        } else {
-            flush_row<T, N>(win, W, rg.acc[N - 1], rg.mref, rg.col_ok, rg.nb + N - 1, lost);
-#pragma unroll
-            for (int b = N - 1; b > 0; --b)
-#pragma unroll
-                for (int a = 0; a < N; ++a) rg.acc[b][a] = rg.acc[b - 1][a] + wy[b] * wx[a];
-#pragma unroll
-            for (int a = 0; a < N; ++a) rg.acc[0][a] = wy[0] * wx[a];
-        }
-        rg.nb = n;
-        return;
-    }
-    // anything else (first node, a jump): flush the whole ring and restart
-    if (rg.live) {
-#pragma unroll
-        for (int b = 0; b < N; ++b) flush_row<T, N>(win, W, rg.acc[b], rg.mref, rg.col_ok, rg.nb + b, lost);
-    }
-#pragma unroll
-    for (int b = 0; b < N; ++b)
-#pragma unroll
-        for (int a = 0; a < N; ++a) rg.acc[b][a] = wy[b] * wx[a];
-    rg.mref = m;
-    rg.nb = n;
-    rg.col_ok = (unsigned)m <= (unsigned)(W.WW - N);
-    rg.live = true;
-}
-
-template <typename T, int N>
-__device__ __forceinline__ void ring_final(T *win, const WinGeom &W, Ring<T, N> &rg, double &lost)
-{
-    if (!rg.live) return;
-#pragma unroll
-    for (int b = 0; b < N; ++b) flush_row<T, N>(win, W, rg.acc[b], rg.mref, rg.col_ok, rg.nb + b, lost);
-    rg.live = false;
-}
-
-// floor of x as a value and as an int without float-to-int conversion instructions:
-// adding 1.5 * 2^(mantissa bits) rounds to an integer held in the low mantissa bits
-// (valid for |x| < 2^51); one compare turns rounding into floor.
-__device__ __forceinline__ void floor_split(double x, double &fl, int &i)
-{
-    const double magic = 6755399441055744.0;   // 1.5 * 2^52
-    const double t = x + magic;
-    double r = t - magic;
-    int k = (int)(__double_as_longlong(t) - 0x4338000000000000LL);
-    if (r > x) {
-        r -= 1.0;
-        k -= 1;
-    }
-    fl = r;
-    i = k;
-}
-
-template <typename T>
-struct ColC {
-    int ui, vi;
-    T uf, vf, cu1, cu2, cv1, cv2;
-};
-
-template <typename T, int BASIS, bool UTERM>
-__device__ __forceinline__ void node_taps(const ColC<T> &c, const RowEntry<T> &r, int colrel,
-                                          int rowrel, T w, int &m, int &n, T *wx, T *wy)
-{
-    using TP = FTaps<T, BASIS>;
-    T fu = c.uf + r.uf;
-    if (UTERM) fu += c.cu1 * r.cy + c.cu2 * r.sy;
-    const T fv = (c.vf + r.vf) + c.cv1 * r.cy + c.cv2 * r.sy;
-    T flu, flv;
-    int iu, iv;
-    floor_split(fu, flu, iu);
-    floor_split(fv, flv, iv);
-    m = colrel + c.ui + r.ui + iu + TP::LO;
-    n = rowrel + c.vi + r.vi + iv + TP::LO;
-    TP::weights(fu - flu, wx);
-    TP::weights(fv - flv, wy);
-#pragma unroll
-    for (int b = 0; b < TP::N; ++b) wy[b] *= w;
-}
 
 // Lambda_x^{-1} (T x = row, T = tridiag(1/6, 2/3, 1/6)) of one row of length L held in
 // shared memory, by one warp. Returns each lane's elements base .. base + per - 1 in v.
@@ -762,26 +531,69 @@ __device__ __forceinline__ void solve_rows_f32(float *win, const WinGeom &W, flo
     }
 }
 
+// Rows of [ja, jb] from which the columns c0 .. c1 (unwrapped, up to nx of them) can reach the widened tile, by one
+// warp: the bounds of the tile's source rectangle for these columns alone. Called where the rectangle is much
+// taller than the tile: strong shear along p, or columns across the period of a force that is not periodic.
+template <typename T>
+__device__ __forceinline__ int2 rows_of_columns(const FusedArgs<T> &A, int c0, int c1, int ja, int jb, int X0, int TXe, int P0,
+                                             int TPe, int D, int R, float Mf, float phif)
+{
+    const Geometry &g = A.g;
+    const float SL = 0.05f;
+    const float EU = fabsf((float)g.KU) * Mf, EV = fabsf((float)g.KV) * Mf, KVM = (float)g.KV * Mf;
+    const float acc_lo = P0 == 0 ? -1e30f : (float)(P0 - R), acc_hi = P0 + TPe == g.np ? 1e30f : (float)(P0 + TPe - 1 + R);
+    const int lane = threadIdx.x & 31;
+    float vcl = 1e30f, vch = -1e30f;
+    for (int c = c0 + lane; c <= c1; c += 32) {
+        const float2 vb = A.vcbf[imod(c, g.nx) / kColBlock];
+        vcl = fminf(vcl, vb.x);
+        vch = fmaxf(vch, vb.y);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        vcl = fminf(vcl, __shfl_xor_sync(0xffffffffu, vcl, o));
+        vch = fmaxf(vch, __shfl_xor_sync(0xffffffffu, vch, o));
+    }
+    int lo = 0x7fffffff, hi = -0x7fffffff;
+    for (int j = ja + lane; j <= jb; j += 32) {
+        const float4 rb = A.rowbf[j];   // u, v, y
+        float tlo = 0.f, thi = 0.f;
+        if (EV > 0.f) {
+            float smin, smax;
+            const float x0f = (float)g.x0, hxf = (float)g.hx, padf = (float)g.a_pad;
+            sin_range32(x0f + c0 * hxf - padf + rb.z + phif, x0f + c1 * hxf + padf + rb.z + phif, smin, smax);
+            tlo = fminf(KVM * smin, KVM * smax);
+            thi = fmaxf(KVM * smin, KVM * smax);
+        }
+        const float vlo = (float)j + rb.y + vcl + tlo - SL, vhi = (float)j + rb.y + vch + thi + SL;
+        const int ia = (int)floorf((float)(X0 - D - R) - rb.x - EU - (float)g.uc_max - SL);
+        const int ib = (int)ceilf((float)(X0 + TXe + D - 1 + R) - rb.x + EU - (float)g.uc_min + SL);
+        if (vhi > acc_lo && vlo < acc_hi && (A.full_row || (c0 <= ib && c1 >= ia))) {
+            lo = min(lo, j);
+            hi = max(hi, j);
+        }
+    }
+    return make_int2(__reduce_min_sync(0xffffffffu, lo), __reduce_max_sync(0xffffffffu, hi));
+}
+
 // ---------------------------------------------------------------------------
 // One destination tile of one simulation (A may live in shared or global memory).
 template <typename T, int BASIS, bool GAL, bool UTERM>
 __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile,
                                            unsigned char *smem_raw)
 {
-    using TP = FTaps<T, BASIS>;
-    constexpr int N = TP::N;
     constexpr int R = (BASIS == VP_BASIS_TENT) ? 1 : 2;
     T *win = reinterpret_cast<T *>(smem_raw);
     T *gcol = win + (size_t)A.ws * (A.tp + 2 * A.Gp);   // [GRows][blockDim] column buffer (Galerkin)
     // row cache: the tile's rows ja .. jb of the push's row table (when they fit)
     RowEntry<T> *rowc = reinterpret_cast<RowEntry<T> *>(gcol + (size_t)GRows<T>::value * blockDim.x);
     __shared__ int s_ia, s_ib, s_ja, s_jb, s_omax;
-    __shared__ double s_part[3][kSumWarps], s_lost[kFusedMaxThreads / 32];
+    __shared__ double s_part[3][kSumWarps], s_lost[kFusedThreads / 32];
     // Thomas pivots of tridiag(1/6, 2/3, 1/6) in T: entry kPivots holds the limit
     constexpr int kPv = sizeof(T) == 4 ? kPiv32 : kPivots;
     __shared__ T piv_cp[kPivots + 1], piv_ib[kPivots + 1];
     __shared__ float2 piv32[kPiv32 + 1];
     __shared__ WalkWin s_win;
+    __shared__ int2 s_rows[kMaxGroups];
     __shared__ T sig_s[kFusedMaxTileP];   // column-sum weights of Lambda_p^{-1} for the tile rows
 
     const Geometry &g = A.g;
@@ -834,7 +646,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         s_ia = s_ja = 0x7fffffff;
         s_ib = s_jb = -0x7fffffff;
         s_omax = 0;
-        if (sizeof(T) == 4) {
+        {
             s_win.WW = W.WW;
             s_win.WH = W.WH;
             s_win.G = G;
@@ -994,15 +806,26 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
             iq = (T)ldexpf(1.f, e2 - 32);
         }
     }
-    __syncthreads();   // the zeroed window, the row table, the pivots
+    // FP32: a thread walks a pair of adjacent columns. The first column of every pair is even where the mesh
+    // allows, so that a pair's source values are one 8-byte load
+    const int ia2 = (nx & 1) == 0 && ib - ia + 2 <= nx ? ia - (ia & 1) : ia;
+    const int wsrc = jb >= ja ? min(ib - ia2 + 1, nx) : 0;
+    const int npair = (wsrc + 1) >> 1, nwp = (npair + 31) >> 5;
+    // a rectangle much taller than the tile: the rows of every warp's columns alone
+    const bool loose = sizeof(T) == 4 && jb - ja + 1 > 2 * TPe + 24 && nwp <= kMaxGroups;
+    if (loose)
+        for (int wi = warp; wi < nwp; wi += nwarps) {
+            const int c0 = ia2 + 64 * wi;
+            int2 r = rows_of_columns<T>(A, c0, min(c0 + 63, ia2 + wsrc - 1), ja, jb, X0, TXe, P0, TPe, D, R, (float)M,
+                                        (float)phi);
+            if (r.x > r.y) r = make_int2(1, 0);
+            if (lane == 0) s_rows[wi] = r;
+        }
+    __syncthreads();   // the zeroed window, the row table, the pivots, the groups' rows
 
     // ---- walk the source columns
     if constexpr (sizeof(T) == 4) {
-        // FP32: items of (pair of adjacent columns, segment of rows). The first column of every pair is
-        // even where the mesh allows, so that a pair's source values are one 8-byte load
-        const int wmax = nx, ia2 = (nx & 1) == 0 && ib - ia + 2 <= nx ? ia - (ia & 1) : ia;
-        const int wsrc = jb >= ja ? min(ib - ia2 + 1, wmax) : 0;
-        const int npair = (wsrc + 1) >> 1;
+        // FP32: items of (pair of adjacent columns, segment of rows)
         const int rows = jb - ja + 1, nseg = min(A.nseg, max(1, rows / kMinSegRows)), len = (rows + nseg - 1) / nseg;
         Walk32 K;
         K.src = A.src;
@@ -1024,10 +847,15 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         K.edge = opaque(K.edge);
         const unsigned gc = smem_addr(gcol) + 8u * tid, gs = 8u * blockDim.x;
         // a warp's lanes share their segment (a warp over two segments runs both, one after the other)
-        const int nwp = (npair + 31) >> 5;
         for (int wi = warp; wi < nwp * nseg; wi += nwarps) {
             const int sg = wi / nwp, q = (wi - sg * nwp) * 32 + lane, ic = ia2 + 2 * q;
-            const int r_lo = ja + sg * len, r_hi = min(jb, r_lo + len - 1);
+            int r_lo = ja + sg * len, r_hi = min(jb, r_lo + len - 1);
+            if (loose) {
+                const int2 r = s_rows[wi - sg * nwp];   // none: (1, 0)
+                const int l = (r.y - r.x + nseg) / nseg;
+                r_lo = r.x + sg * l;
+                r_hi = min(r.y, r_lo + l - 1);
+            }
             if (q >= npair || r_lo > r_hi) continue;
             const int imA = imod(ic, nx), imB = imA + 1 < nx ? imA + 1 : 0;
             // a last pair of one column: its second column takes the weight 0
@@ -1041,156 +869,36 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
                                                     (float)al, (float)be, (float)g.KU, (float)g.KV, gc, gs, lost);
         }
     } else if (jb >= ja) {
-        int wsrc = ib - ia + 1;
-        if (wsrc > nx) wsrc = nx;
-        const T alT = (T)al, beT = (T)be, KU = (T)g.KU, KV = (T)g.KV;
-        const T sixth = T(1) / T(6);
-        for (int cidx = tid; cidx < wsrc; cidx += blockDim.x) {
-            const int ic = ia + cidx;
+        // FP64: items of (column, segment of rows)
+        const int wcol = min(ib - ia + 1, nx);
+        const int rows = jb - ja + 1, nseg = min(A.nseg, max(1, rows / kMinSegRows)), len = (rows + nseg - 1) / nseg;
+        Walk64 K;
+        K.src = A.src;
+        K.nx = nx;
+        K.np = np;
+        K.row = A.row;
+        K.rowc = srow;
+        K.piv_ib = piv_ib;
+        K.piv_cp = piv_cp;
+        K.W = &s_win;
+        K.win = win;
+        K.ws = W.ws;
+        K.lim = W.WH * W.ws;
+        K.WW = W.WW;
+        K.WP0 = W.WP0;
+        K.edge = (P0 == 0 ? 1 : 0) | (P0 + TPe == np ? 2 : 0);
+        const int nw = (wcol + 31) >> 5;
+        for (int wi = warp; wi < nw * nseg; wi += nwarps) {
+            const int sg = wi / nw, q = (wi - sg * nw) * 32 + lane, ic = ia + q;
+            const int r_lo = ja + sg * len, r_hi = min(jb, r_lo + len - 1);
+            if (q >= wcol || r_lo > r_hi) continue;
             const int im = imod(ic, nx);
-            const ColEntry<T> e = A.col[im];
-            ColC<T> cc;
-            cc.ui = e.ui;
-            cc.vi = e.vi;
-            cc.uf = e.uf;
-            cc.vf = e.vf;
-            // sine term: al sin(a + y) + be cos(a + y) = cy (al sa + be ca) + sy (al ca - be sa)
-            const T Pc = alT * e.sa + beT * e.ca, Qc = alT * e.ca - beT * e.sa;
-            cc.cu1 = KU * Pc;
-            cc.cu2 = KU * Qc;
-            cc.cv1 = KV * Pc;
-            cc.cv2 = KV * Qc;
-            const int colrel = ic - W.WX0;
-            const T *src = A.src + im;
-            Ring<T, N> rg;
-            rg.live = false;
-            rg.mref = 0;
-            rg.nb = 0;
-            rg.col_ok = false;
-#pragma unroll
-            for (int q = 0; q < N; ++q)
-#pragma unroll
-                for (int a = 0; a < N; ++a) rg.acc[q][a] = T(0);
-            T wx[N], wy[N];
-            if (!GAL) {
-                // the deposit alone: each chunk of kC source rows is loaded first (all of its loads
-                // in flight, kept in the column buffer), then walked upwards
-                T *gc = gcol + tid;
-                const int nth = blockDim.x;
-                for (int c_lo = ja; c_lo <= jb; c_lo += kC) {
-                    const int c_hi = min(jb, c_lo + kC - 1);
-                    const T *sp = src + (size_t)c_lo * nx;
-                    if (c_hi - c_lo + 1 == kC) {
-#pragma unroll
-                        for (int k = 0; k < kC; ++k) gc[k * nth] = __ldg(sp + (size_t)k * nx);
-                    } else {
-                        for (int k = 0; k <= c_hi - c_lo; ++k) gc[k * nth] = __ldg(sp + (size_t)k * nx);
-                    }
-                    if (rows_cached) {
-#pragma unroll 1
-                        for (int r = c_lo; r <= c_hi; ++r) {
-                            int m, n;
-                            node_taps<T, BASIS, UTERM>(cc, srow[r], colrel, r - W.WP0,
-                                                             gc[(r - c_lo) * nth] * qs, m, n, wx, wy);
-                            ring_add<T, N, 1>(win, W, rg, m, n, wx, wy, lost);
-                        }
-                    } else {
-#pragma unroll 1
-                        for (int r = c_lo; r <= c_hi; ++r) {
-                            int m, n;
-                            node_taps<T, BASIS, UTERM>(cc, A.row[r], colrel, r - W.WP0,
-                                                              gc[(r - c_lo) * nth] * qs, m, n, wx, wy);
-                            ring_add<T, N, 1>(win, W, rg, m, n, wx, wy, lost);
-                        }
-                    }
-                }
-                ring_final<T, N>(win, W, rg, lost);
-            } else {
-                // Lambda_p^{-1} s by the Thomas algorithm, walked downwards in chunks of
-                // kC rows: forward sweep g_j = (s_j - g_{j-1}/6) / beta_j from kHalo rows
-                // below the chunk (or from row 0), kept in the column buffer gcol;
-                // back substitution w_j = g_j - c'_j w_{j+1} continues from the chunk above.
-                T *gc = gcol + tid;
-                const int nth = blockDim.x;
-                T uv = T(0);
-                {
-                    // look-ahead above jb (exact when it reaches the last row)
-                    const int top = min(np - 1, jb + kHalo);
-                    if (top > jb) {
-                        int rr = max(0, jb + 1 - kHalo);
-                        const T *sp = src + (size_t)rr * nx;
-                        T gv = T(0);
-                        for (; rr <= jb; ++rr, sp += nx) gv = (*sp - sixth * gv) * piv_ib[min(rr, kPivots)];
-                        for (; rr <= top; ++rr, sp += nx) {
-                            gv = (*sp - sixth * gv) * piv_ib[min(rr, kPivots)];
-                            gc[(rr - jb - 1) * nth] = gv;
-                        }
-                        for (rr = top; rr > jb; --rr) uv = gc[(rr - jb - 1) * nth] - piv_cp[min(rr, kPivots)] * uv;
-                    }
-                }
-                const T ib_inf = piv_ib[kPivots], cp_inf = piv_cp[kPivots];
-                const T ib6_inf = sixth * ib_inf;
-                for (int c_hi = jb; c_hi >= ja; c_hi -= kC) {
-                    const int c_lo = max(ja, c_hi - kC + 1);
-                    int rr = max(0, c_lo - kHalo);
-                    const T *sp = src + (size_t)rr * nx;
-                    T gv = T(0);
-                    if (c_lo - kHalo > kPivots) {
-                        // far from the first row the pivots have their limits
-                        if (c_hi - c_lo + 1 == kC) {
-                            // whole chunk: warm-up and chunk rows as one unrolled sweep, so that all
-                            // of its loads are in flight before the recurrence needs them
-#pragma unroll
-                            for (int k = 0; k < kHalo + kC; ++k) {
-                                gv = __ldg(sp + (size_t)k * nx) * ib_inf - ib6_inf * gv;
-                                if (k >= kHalo) gc[(k - kHalo) * nth] = gv;
-                            }
-                        } else {
-#pragma unroll 16
-                            for (; rr < c_lo; ++rr, sp += nx) gv = *sp * ib_inf - ib6_inf * gv;
-#pragma unroll 16
-                            for (; rr <= c_hi; ++rr, sp += nx) {
-                                gv = *sp * ib_inf - ib6_inf * gv;
-                                gc[(rr - c_lo) * nth] = gv;
-                            }
-                        }
-                    } else {
-                        for (; rr < c_lo; ++rr, sp += nx) gv = (*sp - sixth * gv) * piv_ib[min(rr, kPivots)];
-                        for (; rr <= c_hi; ++rr, sp += nx) {
-                            gv = (*sp - sixth * gv) * piv_ib[min(rr, kPivots)];
-                            gc[(rr - c_lo) * nth] = gv;
-                        }
-                    }
-                    if (c_lo > kPivots && rows_cached) {
-                        const RowEntry<T> *rp = srow + c_hi;
-#pragma unroll 1
-                        for (int r = c_hi; r >= c_lo; --r, --rp) {
-                            uv = gc[(r - c_lo) * nth] - cp_inf * uv;
-                            int m, n;
-                            node_taps<T, BASIS, UTERM>(cc, *rp, colrel, r - W.WP0, uv * qs, m, n, wx, wy);
-                            ring_add<T, N, -1>(win, W, rg, m, n, wx, wy, lost);
-                        }
-                    } else if (c_lo > kPivots) {
-                        const RowEntry<T> *rp = A.row + c_hi;
-#pragma unroll 1
-                        for (int r = c_hi; r >= c_lo; --r, --rp) {
-                            uv = gc[(r - c_lo) * nth] - cp_inf * uv;
-                            int m, n;
-                            node_taps<T, BASIS, UTERM>(cc, *rp, colrel, r - W.WP0, uv * qs, m, n, wx, wy);
-                            ring_add<T, N, -1>(win, W, rg, m, n, wx, wy, lost);
-                        }
-                    } else {
-                        const RowEntry<T> *rp = A.row + c_hi;
-                        for (int r = c_hi; r >= c_lo; --r, --rp) {
-                            uv = gc[(r - c_lo) * nth] - piv_cp[min(r, kPivots)] * uv;
-                            int m, n;
-                            node_taps<T, BASIS, UTERM>(cc, *rp, colrel, r - W.WP0, uv * qs, m, n, wx, wy);
-                            ring_add<T, N, -1>(win, W, rg, m, n, wx, wy, lost);
-                        }
-                    }
-                }
-                ring_final<T, N>(win, W, rg, lost);
-            }
+            if (rows_cached)
+                walk_col64<BASIS, GAL, UTERM, true>(K, A.col[im], im, ic - W.WX0, r_lo, r_hi, al, be, g.KU, g.KV,
+                                                    gcol + tid, (int)blockDim.x, lost);
+            else
+                walk_col64<BASIS, GAL, UTERM, false>(K, A.col[im], im, ic - W.WX0, r_lo, r_hi, al, be, g.KU, g.KV,
+                                                     gcol + tid, (int)blockDim.x, lost);
         }
     }
     __syncthreads();
@@ -1357,9 +1065,8 @@ __device__ __forceinline__ void finish_step(const FusedArgs<T> &A, unsigned char
     if (threadIdx.x == 0) *A.ticket = 0;
 }
 
-template <typename T, int BASIS, bool GAL, bool UTERM, int MINB>
-__global__ void __launch_bounds__(sizeof(T) == 4 ? kFusedThreads32 : (MINB == 1 ? kFusedMaxThreads : kFusedThreads2),
-                                  sizeof(T) == 4 ? 512 / kFusedThreads32 : MINB)
+template <typename T, int BASIS, bool GAL, bool UTERM>
+__global__ void __launch_bounds__(kFusedThreads, 2)
     step_fused_kernel(const FusedArgs<T> A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1374,7 +1081,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? kFusedThreads32 : (MINB == 1 
 // loop over an atomic counter: inside a loop the compiler kept the arguments of every item live
 // and spilled 400 bytes per thread; one item per CTA spills 60.
 template <typename T, int BASIS, bool GAL, bool UTERM>
-__global__ void __launch_bounds__(kFusedThreads32, 512 / kFusedThreads32)
+__global__ void __launch_bounds__(kFusedThreads, 2)
     step_fused_batch_kernel(const FusedArgs<T> *__restrict__ args, const int *__restrict__ parity,
                             const int *__restrict__ left, const int2 *__restrict__ items, int nitems)
 {
@@ -1410,7 +1117,7 @@ int fused_rowcache_rows(int precision, size_t base_bytes, int ctas)
         if (cudaDeviceGetAttribute(&v, cudaDevAttrReservedSharedMemoryPerBlock, dev) == cudaSuccess) reserved = v;
         cudaFuncAttributes fa;
         const void *k = precision == VP_FP64
-                            ? reinterpret_cast<const void *>(step_fused_kernel<double, VP_BASIS_CUBIC_BSPLINE, true, true, 2>)
+                            ? reinterpret_cast<const void *>(step_fused_kernel<double, VP_BASIS_CUBIC_BSPLINE, true, true>)
                             : reinterpret_cast<const void *>(step_fused_batch_kernel<float, VP_BASIS_CUBIC_BSPLINE, true, true>);
         if (cudaFuncGetAttributes(&fa, k) == cudaSuccess) stat = fa.sharedSizeBytes + 256;
         cudaGetLastError();
@@ -1435,9 +1142,7 @@ cudaError_t launch_step_fused(const FusedArgs<T> &a, int threads, cudaStream_t s
     const bool uterm = a.g.kind == VP_PUSH_FEL_DKD;
 #define VP_LAUNCH_FUSED(B, GL, UT)                                                            \
     do {                                                                                      \
-        auto k = step_fused_kernel<T, B, GL, UT, 2>;                                          \
-        if constexpr (sizeof(T) == 8)                                                         \
-            if (threads > kFusedThreads2) k = step_fused_kernel<T, B, GL, UT, 1>;              \
+        auto k = step_fused_kernel<T, B, GL, UT>;                                             \
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
                                              (int)smem);                                      \
         if (e != cudaSuccess) return e;                                                       \
@@ -1829,7 +1534,7 @@ __device__ __forceinline__ void xsolve_row_regs(T *v, const int base, const int 
 // the next row into its second buffer while it solves the current one.
 template <typename T, int K, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1)
-    xsolve_rows_kernel(const T *__restrict__ r, T *__restrict__ out, int nx, int np,
+    xsolve_rows_kernel(const T *r, T *out, int nx, int np,   // r == out: in place
                        const double *__restrict__ piv, int tx, int tp, int ntx,
                        float *__restrict__ smax_out, unsigned *__restrict__ err, int row_stride, int nbuf)
 {

@@ -91,13 +91,8 @@ struct StepArgs {
 };
 
 // One-pass step kernel (vp_fused.cu): see the description there.
-constexpr int kFusedMaxThreads = 576;   // one CTA per SM (wide tiles)
-constexpr int kFusedThreads2 = 320;     // two CTAs per SM
-#ifndef VP_T
-#define VP_T 256
-#endif
-constexpr int kFusedThreads32 = VP_T;    // FP32: two CTAs of at most 8 warps, so that every SM sub-partition
-                                        // holds 4 warps and a thread may use 128 registers
+constexpr int kFusedThreads = 256;   // two CTAs of at most 8 warps per SM, so that every SM sub-partition
+                                     // holds 4 warps and a thread may use 128 registers
 
 template <typename T>
 struct FusedArgs {
@@ -138,7 +133,7 @@ struct FusedArgs {
     // rows of the push's row table a tile may keep in shared memory (after the window and the
     // column buffer); a tile whose source rows fit reads them there instead of through L1
     int rowcache;
-    // FP32: row segments per pair of source columns. Fixed by the plan (not by the block size), so that a
+    // row segments per pair (FP64: per one) of source columns. Fixed by the plan (not by the block size), so that a
     // simulation's sums are formed in the same pieces alone and in a batch
     int nseg;
     // Galerkin plans with a separate x pass: the tile stores its deposit r = Delta^T w (own

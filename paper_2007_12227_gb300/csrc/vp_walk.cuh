@@ -21,7 +21,7 @@
 // N x N ring per column, acc[b][a] = window row n + b, column m + a; when both nodes land one row
 // further down in the same columns (the common case) the top row leaves the ring for the window.
 // Anything else (first node, a column shift, a jump) adds the ring's rows to the window and restarts
-// it; a node whose footprint leaves the window's columns is added cell by cell.
+// it.
 #pragma once
 
 #include "vp_internal.h"
@@ -120,30 +120,17 @@ __device__ __forceinline__ double lost_cells(const WalkWin *W, const float *v, i
     return s;
 }
 
-// N cells of window row `row` at column m, any of which may lie outside the window: columns wrap in
-// whole-period tiles, rows beyond the open momentum edge count as lost, other cells outside belong to other
-// tiles. Returns the lost weight (window units).
+// Window column of a node's first tap, m, where it lies outside [0, WW - N]. In whole-period tiles it wraps (its
+// N cells then end in the right guard band at the latest, which is folded); in other tiles its cells belong to
+// other tiles or to the guard band, at least N wide, which nobody reads: it is moved into the band.
 template <int N>
-__device__ __forceinline__ double add_cells(const WalkWin *W, unsigned win, int ws4, const float *v, int m, int row)
+__device__ __forceinline__ int fold_col(const WalkWin *W, int m)
 {
-    double lost = 0.0;
-    const bool in = row >= 0 && row < W->WH;
-    const bool gone = !in && ((row + W->WP0 < 0 && (W->edge & 1)) || (row + W->WP0 >= W->np && (W->edge & 2)));
-    if (in || gone) {
-#pragma unroll
-        for (int a = 0; a < N; ++a) {
-            int c = m + a;
-            if (W->full && (c < 0 || c >= W->WW)) {
-                c = (c - W->G) % W->nx;
-                c = W->G + (c < 0 ? c + W->nx : c);
-            }
-            if (c >= 0 && c < W->WW) {
-                if (in) win_add(win + (unsigned)(row * ws4 + 4 * c), v[a]);
-                else lost += lost_cells<1>(W, v + a, c);
-            }
-        }
+    if (W->full) {
+        m = (m - W->G) % W->nx;
+        return W->G + (m < 0 ? m + W->nx : m);
     }
-    return lost;
+    return m < 0 ? 0 : W->WW - N;
 }
 
 // One pair's state. The integer displacement of a node is the low mantissa bits of (fraction + 1.5 2^23)
@@ -155,6 +142,7 @@ struct PairRing {
     int kuA, kuB, kvA, kvB;
     int off;           // window offset (bytes) of column A's leaving row at the next row
     int dBA;           // offset (bytes) of B's cells relative to A's
+    int cA, cB;        // window offset (bytes) of their first columns in window row 0
 };
 constexpr int kRingDead = (int)0x80000000;   // a key no node has
 
@@ -179,11 +167,12 @@ struct Walk32 {
     int edge;              // as in WalkWin
 };
 
-// One row of a pair's rings into the window. Rows outside the window belong to other tiles: their offset is
-// clamped into the window's guard rows, which nobody reads (a predicate on a shared-memory reduction becomes a
-// branch around it). In a tile at an open edge they count as lost, and zeros are added in their place.
+// One row of a pair's rings into the window. Rows outside the window belong to other tiles: they are clamped
+// into the window's guard rows, which nobody reads (a predicate on a shared-memory reduction becomes a
+// branch around it), in their own columns (one common place for them all serialised the warp's additions: 3900
+// cycles a row where strong shear carries most rows outside). In a tile at an open edge they count as lost, and zeros are added in their place.
 template <int N>
-__device__ __forceinline__ void leave_row(const Walk32 &K, const f2_t *acc, int off, int dBA, int mA, int mB, double &lost)
+__device__ __forceinline__ void leave_row(const Walk32 &K, const f2_t *acc, int off, int dBA, int cA, int cB, double &lost)
 {
     float a[N], b[N];
 #pragma unroll
@@ -191,18 +180,19 @@ __device__ __forceinline__ void leave_row(const Walk32 &K, const f2_t *acc, int 
     if (K.edge) {
         const bool inA = (unsigned)off < (unsigned)K.lim, inB = (unsigned)(off + dBA) < (unsigned)K.lim;
         if (!inA) {
-            if (K.edge & (off < 0 ? 1 : 2)) lost += lost_cells<N>(K.W, a, mA);
+            if (K.edge & (off < 0 ? 1 : 2)) lost += lost_cells<N>(K.W, a, cA >> 2);
 #pragma unroll
             for (int q = 0; q < N; ++q) a[q] = 0.f;
         }
         if (!inB) {
-            if (K.edge & (off + dBA < 0 ? 1 : 2)) lost += lost_cells<N>(K.W, b, mB);
+            if (K.edge & (off + dBA < 0 ? 1 : 2)) lost += lost_cells<N>(K.W, b, cB >> 2);
 #pragma unroll
             for (int q = 0; q < N; ++q) b[q] = 0.f;
         }
     }
-    const int top = K.lim - 4 * N;
-    const unsigned pA = K.win + (unsigned)max(0, min(off, top)), pB = K.win + (unsigned)max(0, min(off + dBA, top));
+    const int top = K.lim - K.ws4;
+    const unsigned pA = K.win + (unsigned)max(cA, min(off, top + cA)),
+                   pB = K.win + (unsigned)max(cB, min(off + dBA, top + cB));
 #pragma unroll
     for (int q = 0; q < N; ++q) win_add(pA + 4 * q, a[q]);
 #pragma unroll
@@ -211,11 +201,11 @@ __device__ __forceinline__ void leave_row(const Walk32 &K, const f2_t *acc, int 
 
 // The whole ring, top row first (off: its offset), which leaves it empty.
 template <int N>
-__device__ __forceinline__ void leave_ring(const Walk32 &K, f2_t (&acc)[N][N], int off, int dBA, int mA, int mB, double &lost)
+__device__ __forceinline__ void leave_ring(const Walk32 &K, f2_t (&acc)[N][N], int off, int dBA, int cA, int cB, double &lost)
 {
 #pragma unroll
     for (int k = 0; k < N; ++k, off -= K.ws4) {
-        leave_row<N>(K, acc[N - 1], off, dBA, mA, mB, lost);
+        leave_row<N>(K, acc[N - 1], off, dBA, cA, cB, lost);
 #pragma unroll
         for (int b = N - 1; b > 0; --b)
 #pragma unroll
@@ -320,7 +310,7 @@ __device__ __forceinline__ void walk_pair(const Walk32 &K, const ColEntry<float>
     const float PA = al * eA.sa + be * eA.ca, QA = al * eA.ca - be * eA.sa;
     const float PB = al * eB.sa + be * eB.ca, QB = al * eB.ca - be * eB.sa;
     const f2_t cv1 = f2_pack(KV * PA, KV * PB), cv2 = f2_pack(KV * QA, KV * QB);
-    const f2_t cu1 = f2_pack(KU * PA, KU * PB), cu2 = f2_pack(KU * QA, KU * QB);
+    const f2_t KR = f2_dup(KV != 0.f ? KU / KV : 0.f);   // both are multiples of the same step
     // window column / row of the first tap = key + base (+ the row index)
     const int buA = colrel + eA.ui - kBias + LO, buB = colrel + 1 + eB.ui - kBias + LO;
     const int bvA = eA.vi - kBias + LO - K.WP0, bvB = eB.vi - kBias + LO - K.WP0;
@@ -331,7 +321,7 @@ __device__ __forceinline__ void walk_pair(const Walk32 &K, const ColEntry<float>
     PairRing<N> g;
     g.kuA = kRingDead;
     g.kuB = g.kvA = g.kvB = 0;
-    g.off = g.dBA = 0;
+    g.off = g.dBA = g.cA = g.cB = 0;
 #pragma unroll
     for (int b = 0; b < N; ++b)
 #pragma unroll
@@ -425,8 +415,10 @@ __device__ __forceinline__ void walk_pair(const Walk32 &K, const ColEntry<float>
             rp -= 2;
             const f2_t CY = f2_pack(q1.x, q1.y), SY = f2_pack(q1.z, q1.w);
             f2_t Fu = f2_pack(eA.uf + q0.z, eB.uf + q0.z);
-            if (UTERM) Fu = f2_fma(cu2, SY, f2_fma(cu1, CY, Fu));
-            const f2_t Fv = f2_fma(cv2, SY, f2_fma(cv1, CY, f2_pack(eA.vf + q0.w, eB.vf + q0.w)));
+            f2_t Fv = f2_pack(eA.vf + q0.w, eB.vf + q0.w);
+            // (with UTERM and KU = 0, as a pendulum in a batch, the same bits as without)
+            if (UTERM) Fu = f2_fma(KR, f2_fma(cv2, SY, f2_mul(cv1, CY)), Fu);
+            Fv = f2_fma(cv2, SY, f2_fma(cv1, CY, Fv));
             f2_t bu, bv, wx[N], wy[N];
             pair_weights<N, BASIS>(Fu, bu, wx);
             pair_weights<N, BASIS>(Fv, bv, wy);
@@ -436,41 +428,25 @@ __device__ __forceinline__ void walk_pair(const Walk32 &K, const ColEntry<float>
 #pragma unroll
             for (int b = 0; b < N; ++b) wy[b] = f2_mul(wy[b], w2);
             const int diff = (kuA ^ g.kuA) | (kuB ^ g.kuB) | (kvA ^ g.kvA) | (kvB ^ g.kvB);
-            const int mA = kuA + buA, mB = kuB + buB;
             if (diff != 0) {
                 // not one row further down in the same columns: the ring goes to the window and starts
                 // again (empty, so that the common path below sets it to this node)
-                if (g.kuA != kRingDead) leave_ring<N>(K, g.acc, g.off, g.dBA, g.kuA + buA, g.kuB + buB, lost);
-                const int nA = r + kvA + bvA, nB = r + kvB + bvB;
+                if (g.kuA != kRingDead) leave_ring<N>(K, g.acc, g.off, g.dBA, g.cA, g.cB, lost);
+                int mA = kuA + buA, mB = kuB + buB;
+                const unsigned cmax = (unsigned)(K.WW - N);
+                if ((unsigned)mA > cmax) mA = fold_col<N>(K.W, mA);
+                if ((unsigned)mB > cmax) mB = fold_col<N>(K.W, mB);
                 g.kuA = kuA;
                 g.kuB = kuB;
                 g.kvA = kvA;
                 g.kvB = kvB;
-                g.dBA = (nB - nA) * K.ws4 + 4 * (mB - mA);
-                g.off = (nA + N) * K.ws4 + 4 * mA;
-                const unsigned cmax = (unsigned)(K.WW - N);
-                if ((unsigned)mA > cmax || (unsigned)mB > cmax) {
-                    // outside the window's columns: cell by cell
-#pragma unroll 1
-                    for (int b = 0; b < N; ++b) {
-                        float va[N], vb[N];
-                        f2_t t = wy[0];
-#pragma unroll
-                        for (int q = 1; q < N; ++q) t = b == q ? wy[q] : t;
-#pragma unroll
-                        for (int a = 0; a < N; ++a) f2_unpack(f2_mul(t, wx[a]), va[a], vb[a]);
-                        lost += add_cells<N>(K.W, K.win, K.ws4, va, mA, nA + b);
-                        lost += add_cells<N>(K.W, K.win, K.ws4, vb, mB, nB + b);
-                    }
-#pragma unroll
-                    for (int b = 0; b < N; ++b) wy[b] = 0ull;
-                    g.kuA = kRingDead;
-                    g.off = 0;   // the empty ring's zeros may go anywhere in the window
-                    g.dBA = 4;
-                }
+                g.cA = 4 * mA;
+                g.cB = 4 * mB;
+                g.off = (r + kvA + bvA + N) * K.ws4 + g.cA;
+                g.dBA = (r + kvB + bvB + N) * K.ws4 + g.cB - g.off;
             }
             // the top row leaves, the others move up
-            leave_row<N>(K, g.acc[N - 1], g.off, g.dBA, mA, mB, lost);
+            leave_row<N>(K, g.acc[N - 1], g.off, g.dBA, g.cA, g.cB, lost);
             g.off -= K.ws4;
 #pragma unroll
             for (int b = N - 1; b > 0; --b)
@@ -481,7 +457,7 @@ __device__ __forceinline__ void walk_pair(const Walk32 &K, const ColEntry<float>
         }
         c_hi = c_lo - 1;
     }
-    if (g.kuA != kRingDead) leave_ring<N>(K, g.acc, g.off, g.dBA, g.kuA + buA, g.kuB + buB, lost);
+    leave_ring<N>(K, g.acc, g.off, g.dBA, g.cA, g.cB, lost);
 }
 
 }  // namespace
