@@ -49,7 +49,7 @@ struct Plan {
     // into the state buffer), and a row pass solves Lambda_x along whole rows into the state buffer
     bool x_in_place;
     bool xpass;
-    int xgrid;   // CTAs of the row pass (persistent)
+    int xgrid;   // CTAs of the row pass (persistent); separate filters: 0 where rows are too long for it
     bool rk4;   // FEL with the RK4 integrator: the scatter kernel and stage reductions
     bool septic_gal;   // cubic B-spline basis, Galerkin: 7-band solves after the scatter deposit
     double x7_scale;   // septic x solve: the scale that gives the recursions a unit DC gain
@@ -333,12 +333,19 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
     if (P->xpass && xrow_smem_bytes(opts->precision, grid->nx, P->ntx) > kMaxSmem)
         return fail(msg, VP_ERR_UNSUPPORTED, "the x-solve row pass needs %zu bytes of shared memory",
                     xrow_smem_bytes(opts->precision, grid->nx, P->ntx));
-    P->xgrid = P->xpass ? xrow_grid_size(opts->precision, grid->nx, grid->np, P->ntx) : 0;
+    int xthreads = 0, xchunk = 0;
+    xrow_shape(opts->precision, grid->nx, &xthreads, &xchunk);
+    const bool xfilter = P->galerkin && kernel != VP_KERNEL_FUSED && xthreads > 0 &&
+                         xrow_smem_bytes(opts->precision, grid->nx, 0) <= kMaxSmem;
+    P->xgrid = P->xpass || xfilter
+                   ? xrow_grid_size(opts->precision, grid->nx, grid->np, P->xpass ? P->ntx : 0) : 0;
     P->ntp = (grid->np + tp - 1) / tp;
     P->hist_cap = opts->history_cap ? opts->history_cap : kDefaultHist;
     P->nlost = (kernel == VP_KERNEL_TILED || kernel == VP_KERNEL_FUSED) ? P->ntx * P->ntp : 1;
     P->npart = std::max(std::max(filter_p_blocks(grid->nx, grid->np), P->ntx * P->ntp),
                         fel_partial_blocks(grid->nx, grid->np));
+    // RK4: five sums per block of its stage kernels, in the room for three per part
+    if (P->rk4) P->npart = std::max(P->npart, (5 * rk4_stage_blocks(grid->nx, grid->np) + 2) / 3);
     P->nmblk = moment_blocks(grid->nx, grid->np);
     P->nblk = (grid->nx + kColBlock - 1) / kColBlock;
 
@@ -375,8 +382,8 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
     L.sigma = take(grid->np * sizeof(double));
     // FP32 one-pass plans: max|s| per tile of each state buffer (the fixed-point window scale)
     L.smax = take(kernel == VP_KERNEL_FUSED && sz == 4 ? 2 * (size_t)P->ntx * P->ntp * sizeof(float) : 0);
-    // FEL space charge: half-drift row factors (cos, sin) for the stored state
-    L.rtil = take(P->fel && !P->rk4 && g.sigma2 != 0.0 ? 2 * (size_t)grid->np * sizeof(double) : 0);
+    // FEL space charge, RK4: half-drift row factors (cos, sin) for the stored state
+    L.rtil = take(P->fel && (P->rk4 || g.sigma2 != 0.0) ? 2 * (size_t)grid->np * sizeof(double) : 0);
     // one-pass plans of a push fixed for the whole run: each tile's source rectangle
     L.tsrc = take(kernel == VP_KERNEL_FUSED && !P->fel ? (size_t)P->ntx * P->ntp * sizeof(int4) : 0);
     L.state = take(ST_NSTATE * sizeof(double));
@@ -585,10 +592,10 @@ vp_status do_steps(vp_sim *s, int n, cudaEvent_t *ev = nullptr)
             VP_CUDA(s, cudaMemsetAsync(dst, 0, N * sizeof(T), s->stream));
             if (P.rk4) {
                 VP_CUDA(s, launch_rk4_stages<T>(static_cast<const T *>(src), P.g, s->ptr<double2>(P.L.csx),
-                                                state, part, s->stream));
+                                                s->ptr<double>(P.L.rtil), state, part, s->stream));
                 VP_CUDA(s, launch_rk4_deposit<T>(static_cast<const T *>(src), static_cast<T *>(dst), P.g,
-                                                 s->ptr<double2>(P.L.csx), state, s->ptr<double>(P.L.lost),
-                                                 s->stream));
+                                                 s->ptr<double2>(P.L.csx), s->ptr<double>(P.L.rtil), state,
+                                                 s->ptr<double>(P.L.lost), s->stream));
             } else {
                 VP_CUDA(s, launch_step_scatter<T>(a, s->ptr<double>(P.L.lost), s->stream));
             }
@@ -602,7 +609,7 @@ vp_status do_steps(vp_sim *s, int n, cudaEvent_t *ev = nullptr)
                 float *mout = P.precision == VP_FP32 ? (src == s->f(0) ? m0 + (size_t)P.ntx * P.ntp : m0) : nullptr;
                 VP_CUDA(s, launch_xsolve_rows<T>(P.x_in_place ? static_cast<T *>(dst) : s->ptr<T>(P.L.tmp),
                                                  static_cast<T *>(dst), P.g.nx, P.g.np,
-                                                 s->ptr<double>(P.L.piv), P.tx, P.tp, P.ntx, mout, err,
+                                                 s->ptr<double>(P.L.piv) + kPivXsFused, P.tx, P.tp, P.ntx, mout, err,
                                                  P.xgrid, s->stream));
                 if (e) {
                     VP_CUDA(s, cudaEventRecord(e[2], s->stream));
@@ -611,8 +618,14 @@ vp_status do_steps(vp_sim *s, int n, cudaEvent_t *ev = nullptr)
             }
         } else if (P.galerkin) {
             T *tmp = s->ptr<T>(P.L.tmp);
-            VP_CUDA(s, launch_filter_x<T>(static_cast<const T *>(dst), tmp, P.g.nx, P.g.np,
-                                          s->ptr<double>(P.L.piv), err, s->stream));
+            // rows by the row pass (exact, chunks in registers); longer ones through shared memory
+            if (P.xgrid > 0)
+                VP_CUDA(s, launch_xsolve_rows<T>(static_cast<const T *>(dst), tmp, P.g.nx, P.g.np,
+                                                 s->ptr<double>(P.L.piv) + kPivXsFilter, 1, 1, 0, nullptr, err,
+                                                 P.xgrid, s->stream));
+            else
+                VP_CUDA(s, launch_filter_x<T>(static_cast<const T *>(dst), tmp, P.g.nx, P.g.np,
+                                              s->ptr<double>(P.L.piv), err, s->stream));
             if (e) VP_CUDA(s, cudaEventRecord(e[2], s->stream));
             VP_CUDA(s, launch_filter_p<T>(tmp, static_cast<T *>(dst), P.g.nx, P.g.np,
                                           s->ptr<double>(P.L.piv), s->ptr<double2>(P.L.csx), part,
@@ -869,7 +882,7 @@ vp_status vp_create(const vp_grid *grid, int32_t basis, const vp_pusher *pusher,
     // FEL space charge: cos and sin of the half drift h/2 (delta + p_j), times Lambda_p^{-1}
     // (symmetric) when the stored state is s = Lambda_p w, so that sum_j w_ij f_j = sum_j s_ij rf_j
     std::vector<double> rtil;
-    if (P.fel && !P.rk4 && g.sigma2 != 0.0) {
+    if (P.fel && (P.rk4 || g.sigma2 != 0.0)) {
         rtil.resize(2 * (size_t)g.np);
         for (int j = 0; j < g.np; ++j) {
             const double ph = 0.5 * g.dt * (g.delta + g.p0 + j * g.hp);
@@ -1295,7 +1308,7 @@ vp_status vp_plan(const vp_sim *s, vp_plan_info *out)
     if (P.kernel != VP_KERNEL_FUSED && (P.galerkin || P.septic_gal)) n += 2;
     if (P.septic_gal && P.fel) n += 1;   // FEL partial sums after the septic solves
     if (P.kernel == VP_KERNEL_SCATTER && P.fel && !P.galerkin) n += 1;
-    if (P.rk4) n += 8;   // four stage reductions, each with its amplitude update
+    if (P.rk4) n += 4;   // two reductions for the four stages, each with its amplitude update
     out->launches_per_step = n;
     out->workspace_bytes = (int64_t)P.L.total;
     const bool f64 = P.precision == VP_FP64;

@@ -1535,7 +1535,7 @@ __device__ __forceinline__ void xsolve_row_regs(T *v, const int base, const int 
 template <typename T, int K, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1)
     xsolve_rows_kernel(const T *r, T *out, int nx, int np,   // r == out: in place
-                       const double *__restrict__ piv, int tx, int tp, int ntx,
+                       const double *__restrict__ scale, int tx, int tp, int ntx,
                        float *__restrict__ smax_out, unsigned *__restrict__ err, int row_stride, int nbuf)
 {
     extern __shared__ __align__(16) unsigned char xs_raw[];
@@ -1545,8 +1545,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1)
     constexpr int V = 16 / (int)sizeof(T);
     const int tid = threadIdx.x;
     const bool vec = (nx % V) == 0;   // every row starts 16-byte aligned
-    const T sh = sizeof(T) == 4 ? (T)piv[kPivXsFused] : T(-6) * (T)zconst(1);
-    const T sl = sizeof(T) == 4 ? (T)piv[kPivXsFused + 1] : T(0);
+    const T sh = sizeof(T) == 4 ? (T)scale[0] : T(-6) * (T)zconst(1);
+    const T sl = sizeof(T) == 4 ? (T)scale[1] : T(0);
     const int base = tid * K;
     const int len = max(0, min(K, nx - base));
     // a chunk lies in one tile when the tile width is a multiple of the chunk
@@ -1595,7 +1595,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1)
                 }
         }
         bad |= chk != T(0);
-        if (sizeof(T) == 4 && len > 0) {
+        if (sizeof(T) == 4 && smax_out && len > 0) {
             if (one_tile) {
                 if (m > 0.f) atomicMax(&tmax[base / tx], __float_as_int(m));
             } else {
@@ -1627,7 +1627,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1)
         } else {
             for (int c = tid; c < nx; c += blockDim.x) rout[c] = cur[xrow_idx<T>(c)];
         }
-        if (sizeof(T) == 4) {
+        if (sizeof(T) == 4 && smax_out) {
             int *mo = reinterpret_cast<int *>(smax_out) + (size_t)(row / tp) * ntx;
             for (int k = tid; k < ntx; k += blockDim.x) {
                 const int mk = tmax[k];
@@ -1719,7 +1719,7 @@ int xrow_grid_size(int precision, int nx, int np, int ntx)
 }
 
 template <typename T>
-cudaError_t launch_xsolve_rows(const T *r, T *out, int nx, int np, const double *piv, int tx, int tp,
+cudaError_t launch_xsolve_rows(const T *r, T *out, int nx, int np, const double *scale, int tx, int tp,
                                int ntx, float *smax_out, unsigned *err, int grid, cudaStream_t s)
 {
     const int prec = sizeof(T) == 8 ? VP_FP64 : VP_FP32;
@@ -1735,7 +1735,7 @@ cudaError_t launch_xsolve_rows(const T *r, T *out, int nx, int np, const double 
         if (e != cudaSuccess) return e;
     }
     if (grid <= 0 || grid > np) grid = np;
-    k<<<grid, threads, smem, s>>>(r, out, nx, np, piv, tx, tp, ntx, smax_out, err, stride, nbuf);
+    k<<<grid, threads, smem, s>>>(r, out, nx, np, scale, tx, tp, ntx, smax_out, err, stride, nbuf);
     return cudaGetLastError();
 }
 

@@ -236,10 +236,11 @@ size_t xrow_smem_bytes(int precision, int nx, int ntx);
 int xrow_buffers(int precision, int nx, int ntx);
 int xrow_grid_size(int precision, int nx, int np, int ntx);
 // s' = Lambda_x^{-1} r along every row (cyclic, exact: block-wide carries, no truncation), then
-// FP32: the per-tile max|s'| into smax_out[ntp][ntx] (atomic max over the zeros the step kernel
-// stored); non-finite outputs set ERRF_NONFINITE
+// FP32: scale holds the scale's float pair (device memory), and the per-tile max|s'| goes into
+// smax_out[ntp][ntx] (NULL: not wanted; atomic max over the zeros the step kernel stored); non-finite
+// outputs set ERRF_NONFINITE
 template <typename T>
-cudaError_t launch_xsolve_rows(const T *r, T *out, int nx, int np, const double *piv, int tx, int tp,
+cudaError_t launch_xsolve_rows(const T *r, T *out, int nx, int np, const double *scale, int tx, int tp,
                                int ntx, float *smax_out, unsigned *err, int grid, cudaStream_t s);
 constexpr int kFusedMaxRow = 512; // longest window row one warp solves
 constexpr int kFusedMaxTileP = 256; // tallest tile of the fused kernel
@@ -286,14 +287,14 @@ cudaError_t launch_fel_tilde(const T *state, int nx, int np, const double2 *csx,
                              const double *rs, const double *sig, double *part, cudaStream_t s);
 cudaError_t launch_fel_kick(const double *part, int nparts, double *state, double sigma2,
                             cudaStream_t s);
-// FEL RK4: the four stage reductions and amplitudes (part: rk4_stage_blocks x 3 doubles), and
-// the deposit at the RK4 end points into a zeroed destination
+// FEL RK4: the stage reductions and amplitudes (rt: cos and sin of the half drift per row; part:
+// 5 rk4_stage_blocks doubles), and the deposit at the RK4 end points into a zeroed destination
 int rk4_stage_blocks(int nx, int np);
 template <typename T>
-cudaError_t launch_rk4_stages(const T *w, const Geometry &g, const double2 *csx, double *state,
+cudaError_t launch_rk4_stages(const T *w, const Geometry &g, const double2 *csx, const double *rt, double *state,
                               double *part, cudaStream_t s);
 template <typename T>
-cudaError_t launch_rk4_deposit(const T *src, T *dst, const Geometry &g, const double2 *csx,
+cudaError_t launch_rk4_deposit(const T *src, T *dst, const Geometry &g, const double2 *csx, const double *rt,
                                const double *state, double *lost_acc, cudaStream_t s);
 // init: first bunching after vp_set_f; rk4: A^{n+1} is the RK4 value left in ST_AH
 cudaError_t launch_fel_finalize(const double *part, int nparts, double *state, double *hist,
