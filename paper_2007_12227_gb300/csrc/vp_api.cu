@@ -32,7 +32,7 @@ size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 struct Layout {
     size_t f0, f1, tmp, col, row, rowb, vcb, rowbf, vcbf, csx, ucol, vcol, piv, ldl, sigma, smax, tsrc, rtil,
         state, hist,
-        lost, part, mpart, mout, err, ticket, total;
+        lost, part, mpart, mout, ln, err, ticket, total;
 };
 
 struct Plan {
@@ -392,6 +392,7 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
     L.part = take((size_t)P->npart * 3 * sizeof(double));
     L.mpart = take((size_t)P->nmblk * kNumMoments * sizeof(double));
     L.mout = take(kMoutLen * sizeof(double));
+    L.ln = take(sz == 4 ? kLnTableBytes : 0);
     L.err = take(sizeof(unsigned));
     L.ticket = take(kernel == VP_KERNEL_FUSED ? sizeof(int) : 0);
     L.total = off;
@@ -677,14 +678,23 @@ vp_status do_steps(vp_sim *s, int n, cudaEvent_t *ev = nullptr)
     return VP_OK;
 }
 
-// the initial state block, written by a kernel from its argument (no host buffer to keep alive, so
-// nothing here waits for the stream)
+// The initial state block, written by a kernel from its argument (no host buffer to keep alive, so nothing
+// here waits for the stream), and the zeros of a fresh run in the same launch: they were five memsets, a fifth
+// of the launches that set 40 small simulations' weights.
 struct StateBlock {
     double v[ST_NSTATE];
 };
-__global__ void put_state_kernel(double *dst, StateBlock b)
+struct ZeroRanges {
+    unsigned *p[5];
+    unsigned n[5];   // 4-byte words
+};
+__global__ void reset_kernel(double *dst, StateBlock b, ZeroRanges z)
 {
-    for (int k = threadIdx.x; k < ST_NSTATE; k += blockDim.x) dst[k] = b.v[k];
+    if (blockIdx.x == 0)
+        for (int k = threadIdx.x; k < ST_NSTATE; k += blockDim.x) dst[k] = b.v[k];
+#pragma unroll
+    for (int q = 0; q < 5; ++q)
+        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < z.n[q]; k += gridDim.x * blockDim.x) z.p[q][k] = 0u;
 }
 
 vp_status reset_state(vp_sim *s, const void *w)
@@ -694,12 +704,23 @@ vp_status reset_state(vp_sim *s, const void *w)
     memset(&b, 0, sizeof(b));
     b.v[ST_A_RE] = s->a0_re;
     b.v[ST_A_IM] = s->a0_im;
-    put_state_kernel<<<1, 32, 0, s->stream>>>(s->ptr<double>(P.L.state), b);
+    // FP32 one-pass plans: the map of tile maxima of f0 is zeroed too, for Lambda_p or the maxima pass to fill
+    const bool map = P.kernel == VP_KERNEL_FUSED && P.precision == VP_FP32;
+    ZeroRanges z;
+    memset(&z, 0, sizeof(z));
+    auto zero = [&](int q, size_t off, size_t bytes) {
+        z.p[q] = s->ptr<unsigned>(off);
+        z.n[q] = (unsigned)(bytes / 4);
+    };
+    zero(0, P.L.lost, (size_t)P.nlost * sizeof(double));
+    zero(1, P.L.err, sizeof(unsigned));
+    zero(2, P.L.ticket, P.kernel == VP_KERNEL_FUSED ? sizeof(int) : 0);
+    zero(3, P.L.hist, (size_t)P.hist_cap * 2 * sizeof(double));
+    zero(4, P.L.smax, map ? (size_t)P.ntx * P.ntp * sizeof(float) : 0);
+    const size_t words = std::max(std::max(z.n[0], z.n[3]), z.n[4]);
+    reset_kernel<<<(int)std::min<size_t>(152 * 4, (words + 1023) / 1024 + 1), 256, 0, s->stream>>>(
+        s->ptr<double>(P.L.state), b, z);
     VP_CUDA(s, cudaGetLastError());
-    VP_CUDA(s, cudaMemsetAsync(s->ws + P.L.lost, 0, P.nlost * sizeof(double), s->stream));
-    VP_CUDA(s, cudaMemsetAsync(s->ws + P.L.err, 0, sizeof(unsigned), s->stream));
-    if (P.kernel == VP_KERNEL_FUSED) VP_CUDA(s, cudaMemsetAsync(s->ws + P.L.ticket, 0, sizeof(int), s->stream));
-    VP_CUDA(s, cudaMemsetAsync(s->ws + P.L.hist, 0, (size_t)P.hist_cap * 2 * sizeof(double), s->stream));
     if (P.fel) {
         vp_status st = P.precision == VP_FP64 ? fel_bunching<double>(s, w, 1)
                                               : fel_bunching<float>(s, w, 1);
@@ -789,6 +810,7 @@ vp_status vp_create(const vp_grid *grid, int32_t basis, const vp_pusher *pusher,
     cudaError_t e = build_tables(g, P.precision, s->ws + P.L.col, s->ws + P.L.row,
                                  s->ptr<RowBound>(P.L.rowb), s->ptr<double>(P.L.ucol),
                                  s->ptr<double>(P.L.vcol), s->ptr<double2>(P.L.csx), s->stream);
+    if (e == cudaSuccess && P.precision == VP_FP32) e = build_ln_table(s->ws + P.L.ln, s->stream);
     if (e != cudaSuccess) return cleanup(cuda_fail(nullptr, e, "build_tables"));
     std::vector<double> ucol(g.nx), vcol(g.nx);
     std::vector<RowBound> rowb(g.np);
@@ -1036,15 +1058,15 @@ static vp_status set_f_common(vp_sim *s, const void *src, int32_t dtype, size_t 
         if (P.precision == VP_FP64)
             VP_CUDA(s, launch_lambda_p_mul<double>(static_cast<const double *>(dst),
                                                    static_cast<double *>(s->f(0)), P.g.nx, P.g.np, nullptr,
-                                                   0, 0, 0, 0, s->ptr<unsigned>(P.L.err), s->stream));
+                                                   0, 0, 0, s->ptr<unsigned>(P.L.err), s->stream));
         else
             VP_CUDA(s, launch_lambda_p_mul<float>(static_cast<const float *>(dst),
                                                   static_cast<float *>(s->f(0)), P.g.nx, P.g.np,
-                                                  s->ptr<float>(P.L.smax), P.tx, P.tp, P.ntx, P.ntp,
+                                                  s->ptr<float>(P.L.smax), P.tx, P.tp, P.ntx,
                                                   s->ptr<unsigned>(P.L.err), s->stream));
     } else if (maxima) {
         VP_CUDA(s, launch_tile_max(static_cast<const float *>(s->f(0)), s->ptr<float>(P.L.smax), P.g.nx,
-                                   P.g.np, P.tx, P.tp, P.ntx, P.ntp, s->ptr<unsigned>(P.L.err),
+                                   P.g.np, P.tx, P.tp, P.ntx, s->ptr<unsigned>(P.L.err),
                                    s->stream));
     }
     if (P.fel && !P.rk4 && P.g.sigma2 != 0.0) {
@@ -1202,10 +1224,10 @@ vp_status vp_moments(vp_sim *s, vp_moments_t *out)
     }
     if (P.precision == VP_FP64)
         VP_CUDA(s, launch_moments<double>(static_cast<const double *>(w), P.g,
-                                          s->ptr<double2>(P.L.csx), mpart, P.nmblk, s->stream));
+                                          s->ptr<double2>(P.L.csx), s->ws + P.L.ln, mpart, P.nmblk, s->stream));
     else
         VP_CUDA(s, launch_moments<float>(static_cast<const float *>(w), P.g,
-                                         s->ptr<double2>(P.L.csx), mpart, P.nmblk, s->stream));
+                                         s->ptr<double2>(P.L.csx), s->ws + P.L.ln, mpart, P.nmblk, s->stream));
     // the sums, then the step state and the error flags beside them: one copy to the host
     VP_CUDA(s, launch_moments_finalize(mpart, P.nmblk, s->ptr<double>(P.L.lost), P.nlost, mout,
                                        s->ptr<double>(P.L.state), s->ptr<unsigned>(P.L.err), s->stream));
@@ -1336,7 +1358,6 @@ struct vp_batch {
     int *d_parity;
     int2 *d_items;
     int *d_left;            // per simulation: steps it still takes in the current call
-    BatchFinal *d_fin;
     int nitems, ninst, threads, grid, basis, projection;
     size_t smem;
     cudaGraphExec_t graph;
@@ -1349,7 +1370,7 @@ struct vp_batch {
 namespace {
 
 struct BatchLayout {
-    size_t args, parity, items, left, fin, total;
+    size_t args, parity, items, left, total;
 };
 
 void batch_layout_of(int count, int items, BatchLayout *L);
@@ -1390,7 +1411,6 @@ void batch_layout_of(int count, int items, BatchLayout *L)
     L->parity = take(sizeof(int) * count);
     L->items = take(sizeof(int2) * items);
     L->left = take(sizeof(int) * count);
-    L->fin = take(sizeof(BatchFinal) * count);
     L->total = off;
 }
 
@@ -1406,7 +1426,6 @@ vp_status batch_enqueue_step(vp_batch *b)
     VP_BCUDA(b, launch_step_fused_batch<float>(b->d_args, b->d_parity, b->d_left, b->d_items, b->nitems,
                                                b->basis, b->projection, b->smem, b->threads, b->grid,
                                                b->stream));
-    VP_BCUDA(b, launch_batch_finalize(b->d_fin, b->ninst, b->d_parity, b->d_left, b->stream));
     return VP_OK;
 }
 
@@ -1456,15 +1475,13 @@ vp_status vp_batch_create(vp_sim *const *sims, int32_t count, void *stream, void
     b->d_parity = reinterpret_cast<int *>(b->ws + L.parity);
     b->d_items = reinterpret_cast<int2 *>(b->ws + L.items);
     b->d_left = reinterpret_cast<int *>(b->ws + L.left);
-    b->d_fin = reinterpret_cast<BatchFinal *>(b->ws + L.fin);
     b->nitems = nitems;
     b->ninst = count;
     b->basis = sims[0]->P.g.basis;
     b->projection = sims[0]->P.g.projection;
     b->have_graph = false;
-    // tables: arguments for both buffer parities, the work list (largest tiles first), finals
+    // tables: arguments for both buffer parities, the work list (largest tiles first)
     std::vector<FusedArgs<float>> args(2 * count);
-    std::vector<BatchFinal> fin(count);
     std::vector<int> order(count);
     b->threads = 32;
     b->smem = 0;
@@ -1473,18 +1490,8 @@ vp_status vp_batch_create(vp_sim *const *sims, int32_t count, void *stream, void
         const Plan &P = s->P;
         args[2 * k] = fused_args<float>(s, s->f(0), s->f(1));
         args[2 * k + 1] = fused_args<float>(s, s->f(1), s->f(0));
-        // the batch finishes every simulation's step in its own finalize launch
-        args[2 * k].ticket = nullptr;
-        args[2 * k + 1].ticket = nullptr;
         b->threads = std::max(b->threads, P.threads);
         order[k] = k;
-        fin[k].state = s->ptr<double>(P.L.state);
-        fin[k].part = s->ptr<double>(P.L.part);
-        fin[k].hist = s->ptr<double>(P.L.hist);
-        fin[k].nparts = P.ntx * P.ntp;
-        fin[k].hist_cap = P.hist_cap;
-        fin[k].fel = P.fel ? 1 : 0;
-        fin[k].dt = P.g.dt;
     }
     for (int k = 0; k < count; ++k) {
         const Plan &P = sims[k]->P;
@@ -1504,7 +1511,7 @@ vp_status vp_batch_create(vp_sim *const *sims, int32_t count, void *stream, void
             args[2 * k].rowcache = r;
             args[2 * k + 1].rowcache = r;
         }
-        b->smem += (size_t)rows * sizeof(RowEntry<float>);
+        b->smem = std::max(b->smem + (size_t)rows * sizeof(RowEntry<float>), kFinSmem);
     }
     std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
         const Plan &A = sims[a]->P, &C = sims[c]->P;
@@ -1520,9 +1527,6 @@ vp_status vp_batch_create(vp_sim *const *sims, int32_t count, void *stream, void
                             cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->d_items, items.data(), sizeof(int2) * items.size(),
-                            cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b->d_fin, fin.data(), sizeof(BatchFinal) * fin.size(),
                             cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) {

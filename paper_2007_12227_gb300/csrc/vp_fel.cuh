@@ -13,6 +13,17 @@
 namespace vp {
 
 constexpr int kFinThreads = 256;
+static_assert(kFinSmem == 3 * kFinThreads * sizeof(double), "scratch of fel_finalize_core");
+
+// Amplitude and phase of the kick's sine term, alpha = -Im K, beta = Re K. They only bound the tiles' source
+// windows, with a slack of hundredths of a cell: FP32 (relative error 1e-6 at most, the amplitude rounded up) instead
+// of FP64 hypot and atan2 on the one thread that ends the step.
+__device__ __forceinline__ void store_kick_bounds(double *state)
+{
+    const float re = (float)state[ST_K_RE], im = (float)state[ST_K_IM];
+    state[ST_M] = (double)(hypotf(re, im) * 1.000001f);
+    state[ST_PHI] = (double)atan2f(re, -im);
+}
 
 // Every thread of the block calls it (it synchronises the block), with any block size: the
 // sums run over kFinThreads virtual lanes v (lane v adds the partials v, v + kFinThreads, ...,
@@ -53,8 +64,7 @@ __device__ __forceinline__ void fel_finalize_core(const double *part, int nparts
         // kick amplitude K = A^{1/2} (space charge adds i sigma2 <e^{-i theta~}> afterwards)
         state[ST_K_RE] = state[ST_AH_RE];
         state[ST_K_IM] = state[ST_AH_IM];
-        state[ST_M] = hypot(state[ST_AH_RE], state[ST_AH_IM]);
-        state[ST_PHI] = atan2(state[ST_AH_RE], -state[ST_AH_IM]);
+        store_kick_bounds(state);
         return;
     }
     // DKD: A^{n+1} = A^{n+1/2} + h/2 b^{n+1}; RK4: the stages left A^{n+1} in ST_AH
@@ -67,8 +77,7 @@ __device__ __forceinline__ void fel_finalize_core(const double *part, int nparts
     state[ST_K_RE] = state[ST_AH_RE];
     state[ST_K_IM] = state[ST_AH_IM];
     // sine-term weights of the next push: alpha = -Im K, beta = Re K
-    state[ST_M] = hypot(state[ST_AH_RE], state[ST_AH_IM]);
-    state[ST_PHI] = atan2(state[ST_AH_RE], -state[ST_AH_IM]);
+    store_kick_bounds(state);
     const long step = (long)state[ST_STEP];
     if (hist && hist_cap > 0) {
         const long slot = step % hist_cap;

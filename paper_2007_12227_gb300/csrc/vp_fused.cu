@@ -1035,23 +1035,22 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
     }
 }
 
-// The end of a single simulation's step, in the same launch: each CTA takes a ticket once its
-// tile's partial sums are visible device-wide (thread 0 wrote them, then fences); the CTA that
-// draws the last ticket sees every partial and finishes the step: the FEL field update from all
-// tile partials in the fixed order of fel_finalize_core (the window's shared memory, no longer
-// needed, is its scratch), else the step count. It then resets the counter for the next launch.
-// No CTA waits on another.
+// The end of a simulation's step, in the same launch: each CTA takes a ticket once its tile's partial sums
+// are visible device-wide (they are written and fenced before); the CTA that draws the simulation's last ticket
+// sees every partial and finishes the step: the FEL field update from all tile partials in the fixed order of
+// fel_finalize_core (the window's shared memory, no longer needed, is its scratch), else the step count. It then
+// resets the counter for the next launch. No CTA waits on another. Returns whether this CTA was the last.
 template <typename T>
-__device__ __forceinline__ void finish_step(const FusedArgs<T> &A, unsigned char *smem_raw)
+__device__ __forceinline__ bool finish_step(const FusedArgs<T> &A, unsigned char *smem_raw)
 {
     __shared__ int s_last;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        s_last = atomicAdd(A.ticket, 1) == (int)gridDim.x - 1;
+        s_last = atomicAdd(A.ticket, 1) == A.ntx * A.ntp - 1;
     }
     __syncthreads();
-    if (!s_last) return;
+    if (!s_last) return false;
     __threadfence();
     double *state = const_cast<double *>(A.state);
     if (A.fel_partials) {
@@ -1063,6 +1062,7 @@ __device__ __forceinline__ void finish_step(const FusedArgs<T> &A, unsigned char
         state[ST_TAU] = st * A.g.dt;
     }
     if (threadIdx.x == 0) *A.ticket = 0;
+    return true;
 }
 
 template <typename T, int BASIS, bool GAL, bool UTERM>
@@ -1071,7 +1071,7 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     fused_tile<T, BASIS, GAL, UTERM>(A, blockIdx.x, smem_raw);
-    if (A.ticket) finish_step<T>(A, smem_raw);
+    finish_step<T>(A, smem_raw);
 }
 
 // Batched step: CTA b takes the (instance, tile) item b of the work list (largest tiles first;
@@ -1079,11 +1079,13 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
 // args[2 k + parity[k]] (parity = which buffer holds its current state) and its tile is skipped
 // once the instance has taken its steps (left[k] == 0). One CTA per item rather than a persistent
 // loop over an atomic counter: inside a loop the compiler kept the arguments of every item live
-// and spilled 400 bytes per thread; one item per CTA spills 60.
+// and spilled 400 bytes per thread. The CTA that ends an instance's step (every CTA of it has read
+// parity and left by then) also flips its parity and counts it down: as a launch of its own that took 5 to 8 us a
+// step, against 40 us for the tiles of a dozen served requests.
 template <typename T, int BASIS, bool GAL, bool UTERM>
 __global__ void __launch_bounds__(kFusedThreads, 2)
-    step_fused_batch_kernel(const FusedArgs<T> *__restrict__ args, const int *__restrict__ parity,
-                            const int *__restrict__ left, const int2 *__restrict__ items, int nitems)
+    step_fused_batch_kernel(const FusedArgs<T> *__restrict__ args, int *parity, int *left,
+                            const int2 *__restrict__ items, int nitems)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(16) FusedArgs<T> sA;
@@ -1096,6 +1098,10 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
         reinterpret_cast<int *>(&sA)[k] = reinterpret_cast<const int *>(src)[k];
     __syncthreads();
     fused_tile<T, BASIS, GAL, UTERM>(sA, e.y, smem_raw);
+    if (finish_step<T>(sA, smem_raw) && threadIdx.x == 0) {
+        parity[e.x] ^= 1;
+        left[e.x] -= 1;
+    }
 }
 
 template <typename T>
@@ -1135,8 +1141,7 @@ cudaError_t launch_step_fused(const FusedArgs<T> &a, int threads, cudaStream_t s
     const int wh = a.tp + 2 * a.Gp;
     // the last CTA's field update uses the window memory as its scratch
     const size_t smem_tile = fused_smem_bytes<T>(a.ws, wh, threads, a.rowcache);
-    const size_t smem_fin = (size_t)3 * kFinThreads * sizeof(double);
-    const size_t smem = smem_tile > smem_fin ? smem_tile : smem_fin;
+    const size_t smem = smem_tile > kFinSmem ? smem_tile : kFinSmem;
     const int grid = a.ntx * a.ntp;
     const bool gal = a.g.basis == VP_BASIS_CUBIC_BSPLINE && a.g.projection == VP_PROJ_GALERKIN;
     const bool uterm = a.g.kind == VP_PUSH_FEL_DKD;
@@ -1254,27 +1259,22 @@ static int column_rows(int nx, int np)
     return rows;
 }
 
-cudaError_t launch_tile_max(const float *s, float *map, int nx, int np, int tx, int tp, int ntx,
-                            int ntp, unsigned *err, cudaStream_t st)
+cudaError_t launch_tile_max(const float *s, float *map, int nx, int np, int tx, int tp, int ntx, unsigned *err, cudaStream_t st)
 {
     const int rows = column_rows(nx, np);
-    cudaError_t e = cudaMemsetAsync(map, 0, (size_t)ntx * ntp * sizeof(float), st);
-    if (e != cudaSuccess) return e;
     const dim3 grid((nx + kMulCols - 1) / kMulCols, (np + rows - 1) / rows);
     tile_max_kernel<<<grid, kMulCols, 0, st>>>(s, reinterpret_cast<unsigned *>(map), nx, np, rows, tx, tp, ntx, err);
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_lambda_p_mul(const T *w, T *s, int nx, int np, float *map, int tx, int tp, int ntx, int ntp,
+cudaError_t launch_lambda_p_mul(const T *w, T *s, int nx, int np, float *map, int tx, int tp, int ntx,
                                 unsigned *err, cudaStream_t st)
 {
     const int rows = column_rows(nx, np);
     const dim3 grid((nx + kMulCols - 1) / kMulCols, (np + rows - 1) / rows);
     if ((np + 63) / 64 > 65535) return cudaErrorInvalidConfiguration;
     if (map) {
-        cudaError_t e = cudaMemsetAsync(map, 0, (size_t)ntx * ntp * sizeof(float), st);
-        if (e != cudaSuccess) return e;
         lambda_p_mul_kernel<T, true><<<grid, kMulCols, 0, st>>>(w, s, nx, np, rows, reinterpret_cast<unsigned *>(map), tx,
                                                                 tp, ntx, err);
     } else {
@@ -1284,7 +1284,7 @@ cudaError_t launch_lambda_p_mul(const T *w, T *s, int nx, int np, float *map, in
 }
 
 template <typename T>
-cudaError_t launch_step_fused_batch(const FusedArgs<T> *args, const int *parity, const int *left,
+cudaError_t launch_step_fused_batch(const FusedArgs<T> *args, int *parity, int *left,
                                     const int2 *items, int nitems, int basis, int projection,
                                     size_t smem, int threads, int grid, cudaStream_t s)
 {
@@ -1744,16 +1744,16 @@ template cudaError_t launch_xsolve_rows<float>(const float *, float *, int, int,
 template cudaError_t launch_xsolve_rows<double>(const double *, double *, int, int, const double *, int,
                                                 int, int, float *, unsigned *, int, cudaStream_t);
 
-template cudaError_t launch_step_fused_batch<float>(const FusedArgs<float> *, const int *, const int *,
+template cudaError_t launch_step_fused_batch<float>(const FusedArgs<float> *, int *, int *,
                                                     const int2 *, int, int, int, size_t, int, int,
                                                     cudaStream_t);
 template size_t fused_smem_bytes<float>(int, int, int, int);
 template size_t fused_smem_bytes<double>(int, int, int, int);
 template cudaError_t launch_step_fused<float>(const FusedArgs<float> &, int, cudaStream_t);
 template cudaError_t launch_step_fused<double>(const FusedArgs<double> &, int, cudaStream_t);
-template cudaError_t launch_lambda_p_mul<float>(const float *, float *, int, int, float *, int, int, int, int,
+template cudaError_t launch_lambda_p_mul<float>(const float *, float *, int, int, float *, int, int, int,
                                                 unsigned *, cudaStream_t);
-template cudaError_t launch_lambda_p_mul<double>(const double *, double *, int, int, float *, int, int, int, int,
+template cudaError_t launch_lambda_p_mul<double>(const double *, double *, int, int, float *, int, int, int,
                                                  unsigned *, cudaStream_t);
 
 }  // namespace vp

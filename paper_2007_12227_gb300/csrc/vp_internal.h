@@ -91,6 +91,7 @@ struct StepArgs {
 };
 
 // One-pass step kernel (vp_fused.cu): see the description there.
+constexpr size_t kFinSmem = 3 * 256 * sizeof(double);   // scratch of the field update in the step kernel's last CTA
 constexpr int kFusedThreads = 256;   // two CTAs of at most 8 warps per SM, so that every SM sub-partition
                                      // holds 4 warps and a thread may use 128 registers
 
@@ -205,22 +206,13 @@ int fused_rowcache_rows(int precision, size_t base_bytes, int ctas);
 // CTAs of the FP32 batched step kernel per SM at this shared memory and block size (0: unknown)
 int fused_batch_blocks_per_sm(int basis, int projection, size_t smem, int threads);
 // one CTA per item (grid >= nitems; grid <= 0: set the shared-memory attribute only);
-// left[k]: steps simulation k still takes in this call; its items are skipped at 0
+// left[k]: steps simulation k still takes in this call; its items are skipped at 0. The step ends every
+// simulation it advances: field update or step count, parity[k] flipped, left[k] counted down
 template <typename T>
-cudaError_t launch_step_fused_batch(const FusedArgs<T> *args, const int *parity, const int *left,
+cudaError_t launch_step_fused_batch(const FusedArgs<T> *args, int *parity, int *left,
                                     const int2 *items, int nitems, int basis, int projection,
                                     size_t smem, int threads, int grid, cudaStream_t s);
 
-// per-instance end-of-step work of a batch: FEL field update, or the step counter
-struct BatchFinal {
-    double *state;
-    const double *part;
-    double *hist;
-    int nparts, hist_cap, fel;
-    double dt;
-};
-// finishes the step of every simulation with left[k] > 0, flips its parity, decrements left[k]
-cudaError_t launch_batch_finalize(const BatchFinal *fin, int ninst, int *parity, int *left, cudaStream_t s);
 // device bytes of a batch of `count` simulations with `items` tiles in all
 size_t batch_workspace_bytes(int count, int items);
 constexpr int fused_halo(int precision) { return precision == VP_FP64 ? 28 : 16; }
@@ -246,11 +238,11 @@ constexpr int kFusedMaxRow = 512; // longest window row one warp solves
 constexpr int kFusedMaxTileP = 256; // tallest tile of the fused kernel
 // s = Lambda_p w; map (may be NULL): max|s| per tile as launch_tile_max gives it
 template <typename T>
-cudaError_t launch_lambda_p_mul(const T *w, T *s, int nx, int np, float *map, int tx, int tp, int ntx, int ntp,
+cudaError_t launch_lambda_p_mul(const T *w, T *s, int nx, int np, float *map, int tx, int tp, int ntx,
                                 unsigned *err, cudaStream_t st);
-// max|s| of an FP32 state over each tile x tile_p tile into map[ntp][ntx]; non-finite -> err
-cudaError_t launch_tile_max(const float *s, float *map, int nx, int np, int tx, int tp, int ntx,
-                            int ntp, unsigned *err, cudaStream_t st);
+// max|s| of an FP32 state over each tile x tile_p tile into the zeroed map[ntp][ntx]; non-finite -> infinity, err
+cudaError_t launch_tile_max(const float *s, float *map, int nx, int np, int tx, int tp, int ntx, unsigned *err,
+                            cudaStream_t st);
 
 template <typename T>
 cudaError_t launch_filter_x(const T *in, T *out, int nx, int np, const double *piv, unsigned *err,
@@ -301,8 +293,11 @@ cudaError_t launch_fel_finalize(const double *part, int nparts, double *state, d
                                 int hist_cap, double dt, int init, cudaStream_t s, int rk4 = 0);
 cudaError_t launch_count_step(double *state, double dt, cudaStream_t s);
 
+// ln: the table of ln of FP32 weights that build_ln_table writes (kLnTableBytes)
+constexpr size_t kLnTableBytes = 512 * 16 + 256 * 8;
+cudaError_t build_ln_table(void *ln, cudaStream_t s);
 template <typename T>
-cudaError_t launch_moments(const T *w, const Geometry &g, const double2 *csx, double *part,
+cudaError_t launch_moments(const T *w, const Geometry &g, const double2 *csx, const void *ln, double *part,
                            int nblocks, cudaStream_t s);
 int moment_blocks(int nx, int np);
 // out: the kNumMoments sums and the lost weight, the step state from kMoutState on, then the error flags

@@ -128,8 +128,7 @@ __global__ void fel_kick_kernel(const double *__restrict__ part, int nparts, dou
     const double kr = state[ST_AH_RE] - sigma2 * bt_im, ki = state[ST_AH_IM] + sigma2 * bt_re;
     state[ST_K_RE] = kr;
     state[ST_K_IM] = ki;
-    state[ST_M] = hypot(kr, ki);
-    state[ST_PHI] = atan2(kr, -ki);
+    store_kick_bounds(state);
 }
 
 // FEL field update from per-block partial sums (run by one block of kFinThreads threads)
@@ -146,26 +145,6 @@ __global__ void fel_finalize_kernel(const double *__restrict__ part, int nparts,
     fel_finalize_block(part, nparts, state, hist, hist_cap, dt, init, rk4);
 }
 
-// end of a batched step: block k finishes instance k, flips its buffer parity and counts down
-// the steps it still takes in this call (instances already at zero are left alone)
-__global__ void batch_finalize_kernel(const BatchFinal *__restrict__ fin, int *parity, int *left)
-{
-    if (left[blockIdx.x] <= 0) return;
-    const BatchFinal f = fin[blockIdx.x];
-    if (f.fel) {
-        fel_finalize_block(f.part, f.nparts, f.state, f.hist, f.hist_cap, f.dt, 0);
-    } else if (threadIdx.x == 0) {
-        const double st = f.state[ST_STEP] + 1.0;
-        f.state[ST_STEP] = st;
-        f.state[ST_TAU] = st * f.dt;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        parity[blockIdx.x] ^= 1;
-        left[blockIdx.x] -= 1;
-    }
-}
-
 // plain step counter for non-FEL sims
 __global__ void count_step_kernel(double *state, double dt)
 {
@@ -175,7 +154,7 @@ __global__ void count_step_kernel(double *state, double dt)
 }
 
 // Moments. Bound by the FP64 pipe (2 operations per clock and SM on this GPU), not by memory: 62 FP64
-// operations a node took 0.45 ms for 2048 x 2048 (0.28 ms now, the final sums 12 us against 153 in one thread
+// operations a node took 0.45 ms for 2048 x 2048 (REPLACEMOM now, the final sums 12 us against 153 in one thread
 // each). A warp therefore walks 32 columns through a chunk of rows and
 // keeps per column only the sums over p (w, w p, w p^2: everything else of a node's moments is a factor of its
 // column), the entropy, and the negative and the trapped weight: about a dozen.
@@ -184,18 +163,21 @@ __global__ void count_step_kernel(double *state, double dt)
 // ln w = (e ln 2 + ln c) + ln(1 + u), the series of ln(1 + u) cut after u^5 / 5 (the next term is below 2^-62). 1 / c
 // is rounded, so ln c in the table is minus the log of that rounded value: u carries one rounding, of order 2^-53.
 constexpr int kLnBits = 9, kLnTab = 1 << kLnBits;
-struct LnTable {
+struct alignas(16) LnTable {
     double2 c[kLnTab];   // rounded 1 / c, and -ln of it
     double e[256];       // (e - 127) ln 2
 };
 
-__device__ __forceinline__ void ln_table(LnTable &t)
+static_assert(sizeof(LnTable) == kLnTableBytes, "room for the table in the workspace");
+
+__global__ void ln_table_kernel(LnTable *t)
 {
-    for (int k = threadIdx.x; k < kLnTab; k += blockDim.x) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < kLnTab) {
         const double ic = 1.0 / (1.0 + (k + 0.5) / kLnTab);
-        t.c[k] = make_double2(ic, -log(ic));
+        t->c[k] = make_double2(ic, -log(ic));
     }
-    for (int k = threadIdx.x; k < 256; k += blockDim.x) t.e[k] = (k - 127) * 0.693147180559945309417;
+    if (k < 256) t->e[k] = (k - 127) * 0.693147180559945309417;
 }
 
 // conversion by integer operations where it can be (a conversion instruction runs at the FP64 rate)
@@ -227,8 +209,9 @@ __device__ __forceinline__ double ln_of(double w, const LnTable &) { return log(
 // rows of a warp's chunk and the chunks of a column (the same on the host and in the kernel)
 __host__ __device__ __forceinline__ int moment_rows(int nx, int np)
 {
-    // about 8 warps on each of the 8 blocks of an SM; at least 8 rows, so that the column factors are spread
-    const long long strips = (nx + 31) / 32, want = 152LL * 8 * 8;
+    // as many warps as the chip holds (16 an SM); at least 8 rows, over which a column's factors and the block's
+    // final sums are spread
+    const long long strips = (nx + 31) / 32, want = 152LL * 16;
     const long long chunks = want / strips < 1 ? 1 : want / strips;
     const long long rows = (np + chunks - 1) / chunks;
     return rows < 8 ? 8 : (int)rows;
@@ -236,11 +219,13 @@ __host__ __device__ __forceinline__ int moment_rows(int nx, int np)
 
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
-    moments_kernel(const T *__restrict__ w, Geometry g, const double2 *__restrict__ csx, double *part)
+    moments_kernel(const T *__restrict__ w, Geometry g, const double2 *__restrict__ csx, const void *ln, double *part)
 {
     __shared__ double s_red[kNumMoments][kRedThreads / 32];
     __shared__ LnTable s_ln;
-    if (sizeof(T) == 4) ln_table(s_ln);
+    if (sizeof(T) == 4)
+        for (int k = threadIdx.x; k < (int)(sizeof(LnTable) / 16); k += kRedThreads)
+            reinterpret_cast<int4 *>(&s_ln)[k] = __ldg(static_cast<const int4 *>(ln) + k);
     __syncthreads();
     const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
     double acc[kNumMoments];
@@ -415,12 +400,6 @@ cudaError_t launch_fel_finalize(const double *part, int nparts, double *state, d
     return cudaGetLastError();
 }
 
-cudaError_t launch_batch_finalize(const BatchFinal *fin, int ninst, int *parity, int *left, cudaStream_t s)
-{
-    batch_finalize_kernel<<<ninst, kRedThreads, 0, s>>>(fin, parity, left);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_count_step(double *state, double dt, cudaStream_t s)
 {
     count_step_kernel<<<1, 1, 0, s>>>(state, dt);
@@ -436,10 +415,16 @@ int moment_blocks(int nx, int np)
 }
 
 template <typename T>
-cudaError_t launch_moments(const T *w, const Geometry &g, const double2 *csx, double *part,
+cudaError_t launch_moments(const T *w, const Geometry &g, const double2 *csx, const void *ln, double *part,
                            int nblocks, cudaStream_t s)
 {
-    moments_kernel<T><<<nblocks, kRedThreads, 0, s>>>(w, g, csx, part);
+    moments_kernel<T><<<nblocks, kRedThreads, 0, s>>>(w, g, csx, ln, part);
+    return cudaGetLastError();
+}
+
+cudaError_t build_ln_table(void *ln, cudaStream_t s)
+{
+    ln_table_kernel<<<(kLnTab + 127) / 128, 128, 0, s>>>(static_cast<LnTable *>(ln));
     return cudaGetLastError();
 }
 
@@ -463,9 +448,9 @@ template cudaError_t launch_fel_partials<float>(const float *, int, int, const d
                                                 cudaStream_t);
 template cudaError_t launch_fel_partials<double>(const double *, int, int, const double2 *,
                                                  double *, cudaStream_t);
-template cudaError_t launch_moments<float>(const float *, const Geometry &, const double2 *,
+template cudaError_t launch_moments<float>(const float *, const Geometry &, const double2 *, const void *,
                                            double *, int, cudaStream_t);
-template cudaError_t launch_moments<double>(const double *, const Geometry &, const double2 *,
+template cudaError_t launch_moments<double>(const double *, const Geometry &, const double2 *, const void *,
                                             double *, int, cudaStream_t);
 template cudaError_t launch_convert<float, double>(const float *, double *, size_t, cudaStream_t);
 template cudaError_t launch_convert<double, float>(const double *, float *, size_t, cudaStream_t);
