@@ -578,6 +578,15 @@ vp_status do_steps(vp_sim *s, int n, cudaEvent_t *ev = nullptr)
     double *part = s->ptr<double>(P.L.part);
     double *state = s->ptr<double>(P.L.state);
     unsigned *err = s->ptr<unsigned>(P.L.err);
+    // a step's launch may begin while the one before it ends, except under events between the phases and in a
+    // stream that is being captured (a captured step is an ordinary kernel node)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    bool ahead = ev == nullptr;
+    if (ahead && cudaStreamIsCapturing(s->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        ahead = false;
+    }
+    ahead = ahead && cap == cudaStreamCaptureStatusNone;
     for (int k = 0; k < n; ++k) {
         cudaEvent_t *e = ev ? ev + (size_t)k * (VP_NPHASES + 1) : nullptr;
         if (e) VP_CUDA(s, cudaEventRecord(e[0], s->stream));
@@ -586,7 +595,7 @@ vp_status do_steps(vp_sim *s, int n, cudaEvent_t *ev = nullptr)
         if (P.kernel == VP_KERNEL_FUSED) {
             // separate x pass: the tiles store the deposit into tmp (or dst), the row pass solves it into dst
             void *tile_dst = P.xpass && !P.x_in_place ? static_cast<void *>(s->ptr<T>(P.L.tmp)) : dst;
-            VP_CUDA(s, launch_step_fused<T>(fused_args<T>(s, src, tile_dst), P.threads, s->stream));
+            VP_CUDA(s, launch_step_fused<T>(fused_args<T>(s, src, tile_dst), P.threads, ahead, s->stream));
         } else if (P.kernel == VP_KERNEL_TILED) {
             VP_CUDA(s, launch_step_tiled<T>(a, s->stream));
         } else {
@@ -611,7 +620,7 @@ vp_status do_steps(vp_sim *s, int n, cudaEvent_t *ev = nullptr)
                 VP_CUDA(s, launch_xsolve_rows<T>(P.x_in_place ? static_cast<T *>(dst) : s->ptr<T>(P.L.tmp),
                                                  static_cast<T *>(dst), P.g.nx, P.g.np,
                                                  s->ptr<double>(P.L.piv) + kPivXsFused, P.tx, P.tp, P.ntx, mout, err,
-                                                 P.xgrid, s->stream));
+                                                 P.xgrid, ahead, s->stream));
                 if (e) {
                     VP_CUDA(s, cudaEventRecord(e[2], s->stream));
                     VP_CUDA(s, cudaEventRecord(e[3], s->stream));
@@ -623,7 +632,7 @@ vp_status do_steps(vp_sim *s, int n, cudaEvent_t *ev = nullptr)
             if (P.xgrid > 0)
                 VP_CUDA(s, launch_xsolve_rows<T>(static_cast<const T *>(dst), tmp, P.g.nx, P.g.np,
                                                  s->ptr<double>(P.L.piv) + kPivXsFilter, 1, 1, 0, nullptr, err,
-                                                 P.xgrid, s->stream));
+                                                 P.xgrid, ahead, s->stream));
             else
                 VP_CUDA(s, launch_filter_x<T>(static_cast<const T *>(dst), tmp, P.g.nx, P.g.np,
                                               s->ptr<double>(P.L.piv), err, s->stream));

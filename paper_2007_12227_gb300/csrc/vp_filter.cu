@@ -113,7 +113,14 @@ __global__ void filter_x_kernel(const T *__restrict__ in, T *__restrict__ out, i
     (void)err;
 }
 
-constexpr int kPThreads = 128;   // columns per block
+constexpr int kPThreads = 128;   // columns per block, at most
+// A mesh of few blocks runs one warp per block: the chip's SMs share them evenly (FP64 256 x 512: 32 blocks of 4 warps
+// took 31 us, each warp's operations waiting for the others' in the FP64 pipe of its SM).
+static int filter_p_threads(int nx, int np)
+{
+    const long blocks = (long)((nx + kPThreads - 1) / kPThreads) * ((np + 31) / 32);
+    return blocks < 152 * 4 ? 32 : kPThreads;
+}
 constexpr int kPChunk = 32;      // rows per chunk, kept in registers
 
 // piv[2 r] = c'_r (super-diagonal factor), piv[2 r + 1] = 1 / beta_r, r < kPivots;
@@ -130,7 +137,7 @@ constexpr int kPChunk = 32;      // rows per chunk, kept in registers
 template <typename T, bool FAR>
 __device__ __forceinline__ bool solve_p_chunk(const T *__restrict__ in, T *__restrict__ out, int nx, int np, int col,
                                               int s, T ib_inf, T cp_inf, const T *s_cp, const T *s_ib, bool want_part,
-                                              DSum<T> &wacc)
+                                              DSum<T> *wacc)
 {
     constexpr int K = Trunc<T>::K, C = kPChunk;
     const T sixth = (T)(1.0 / 6.0);
@@ -142,10 +149,16 @@ __device__ __forceinline__ bool solve_p_chunk(const T *__restrict__ in, T *__res
         const int r = s - K + k;
         return r >= 0 && r < np ? __ldg(src + (size_t)r * pitch) : T(0);
     };
+    // FP64: one dependent operation a row (about 75 clocks each on this GPU) instead of two; FP32 keeps the form whose
+    // gain the x solve's scale makes up for
+    auto row_step = [&](T x, T g, T ib) -> T {
+        if constexpr (sizeof(T) == 8) return fma(-(sixth * ib), g, x * ib);
+        return (x - sixth * g) * ib;
+    };
     auto step = [&](int k, T x, T g) -> T {
-        if (FAR) return (x - sixth * g) * ib_inf;
+        if (FAR) return row_step(x, g, ib_inf);
         const int r = s - K + k;
-        return r >= 0 && r < np ? (x - sixth * g) * s_ib[min(r, kPivots)] : g;
+        return r >= 0 && r < np ? row_step(x, g, s_ib[min(r, kPivots)]) : g;
     };
     constexpr int F = 16;   // loads in flight
     T x[F], gc[C], g = T(0);
@@ -178,7 +191,7 @@ __device__ __forceinline__ bool solve_p_chunk(const T *__restrict__ in, T *__res
             w = gc[k] - (FAR ? cp_inf : s_cp[min(s + k, kPivots)]) * w;
             dst[(size_t)(unsigned)k * pitch] = w;
             chk = fma(w, T(0), chk);
-            if (want_part) wacc.add(w);
+            if (want_part) wacc[k & 3].add(w);   // four chains of the compensated sum
         }
     }
     return chk != T(0);
@@ -194,18 +207,18 @@ __global__ void __launch_bounds__(kPThreads)
     __shared__ T s_cp[kPivots + 1], s_ib[kPivots + 1];
     constexpr int K = Trunc<T>::K;
     const int tid = threadIdx.x, lane = tid & 31, wy = tid >> 5;
-    const int cblk = (nx + kPThreads - 1) / kPThreads;   // blocks of columns, fastest
-    const int col = (int)(blockIdx.x % cblk) * kPThreads + tid;
+    const int nt = blockDim.x, cblk = (nx + nt - 1) / nt;   // blocks of columns, fastest
+    const int col = (int)(blockIdx.x % cblk) * nt + tid;
     const int s = (int)(blockIdx.x / cblk) * kPChunk;
     const bool far = s - K >= kPivots && s + kPChunk + K <= np;
     if (!far) {
-        for (int k = tid; k <= kPivots; k += kPThreads) {
+        for (int k = tid; k <= kPivots; k += nt) {
             s_cp[k] = (T)piv[2 * k];
             s_ib[k] = (T)piv[2 * k + 1];
         }
         __syncthreads();
     }
-    DSum<T> wacc;
+    DSum<T> wacc[4];
     bool bad = false;
     if (col < nx) {
         const T cp_inf = (T)piv[2 * kPivots], ib_inf = (T)piv[2 * kPivots + 1];
@@ -216,7 +229,7 @@ __global__ void __launch_bounds__(kPThreads)
     if (!want_part) return;
     double pw = 0.0, pc = 0.0, ps = 0.0;
     if (col < nx) {
-        pw = wacc.value();
+        pw = (wacc[0].value() + wacc[1].value()) + (wacc[2].value() + wacc[3].value());
         const double2 t = csx[col];
         pc = pw * t.x;
         ps = pw * t.y;
@@ -232,7 +245,7 @@ __global__ void __launch_bounds__(kPThreads)
         const size_t b = blockIdx.x;
         for (int q = 0; q < 3; ++q) {
             double t = 0.0;
-            for (int w = 0; w < kPThreads / 32; ++w) t += s_red[q][w];
+            for (int w = 0; w < nt / 32; ++w) t += s_red[q][w];
             part[3 * b + q] = t;
         }
     }
@@ -395,7 +408,8 @@ template cudaError_t launch_filter_p7<double>(const double *, double *, int, int
 
 int filter_p_blocks(int nx, int np)
 {
-    return ((nx + kPThreads - 1) / kPThreads) * ((np + kPChunk - 1) / kPChunk);
+    const int nt = filter_p_threads(nx, np);
+    return ((nx + nt - 1) / nt) * ((np + kPChunk - 1) / kPChunk);
 }
 
 template <typename T>
@@ -403,7 +417,7 @@ cudaError_t launch_filter_p(const T *in, T *out, int nx, int np, const double *p
                             const double2 *csx, double *part, int want_part, unsigned *err,
                             cudaStream_t s)
 {
-    filter_p_kernel<T><<<filter_p_blocks(nx, np), kPThreads, 0, s>>>(in, out, nx, np, piv, csx, part, want_part, err);
+    filter_p_kernel<T><<<filter_p_blocks(nx, np), filter_p_threads(nx, np), 0, s>>>(in, out, nx, np, piv, csx, part, want_part, err);
     return cudaGetLastError();
 }
 

@@ -195,8 +195,9 @@ cudaError_t launch_step_scatter(const StepArgs<T> &a, double *lost_acc, cudaStre
 template <typename T>
 size_t tiled_smem_bytes(int tx, int tp);
 
+// ahead: the launch may begin while the one before it in the stream ends (programmatic dependent launch)
 template <typename T>
-cudaError_t launch_step_fused(const FusedArgs<T> &a, int threads, cudaStream_t s);
+cudaError_t launch_step_fused(const FusedArgs<T> &a, int threads, bool ahead, cudaStream_t s);
 // dynamic shared memory of the one-pass kernel: window (ws x wh), column buffer, row cache
 template <typename T>
 size_t fused_smem_bytes(int ws, int wh, int threads, int rowcache = 0);
@@ -233,7 +234,7 @@ int xrow_grid_size(int precision, int nx, int np, int ntx);
 // outputs set ERRF_NONFINITE
 template <typename T>
 cudaError_t launch_xsolve_rows(const T *r, T *out, int nx, int np, const double *scale, int tx, int tp,
-                               int ntx, float *smax_out, unsigned *err, int grid, cudaStream_t s);
+                               int ntx, float *smax_out, unsigned *err, int grid, bool ahead, cudaStream_t s);
 constexpr int kFusedMaxRow = 512; // longest window row one warp solves
 constexpr int kFusedMaxTileP = 256; // tallest tile of the fused kernel
 // s = Lambda_p w; map (may be NULL): max|s| per tile as launch_tile_max gives it

