@@ -37,6 +37,7 @@ UNIT = "node-updates/s"
 FALLBACK_HBM_GBS = 6800.0
 # sources of the one-pass step kernel: the committed ncu traffic applies only to these bytes
 FUSED_SOURCES = ["paper_2007_12227_gb300/csrc/vp_fused.cu", "paper_2007_12227_gb300/csrc/vp_internal.h",
+                 "paper_2007_12227_gb300/csrc/vp_walk.cuh", "paper_2007_12227_gb300/csrc/vp_walk64.cuh",
                  "paper_2007_12227_gb300/csrc/vp_sum.cuh", "paper_2007_12227_gb300/csrc/vp_fel.cuh"]
 
 
