@@ -8,8 +8,9 @@
 // row's push entry, the loop and the test for the common case are paid once for two nodes. Two CTAs of 8
 // warps share an SM (4 warps a sub-partition, 128 registers a thread). Measured on the 4096 x 4096
 // pendulum step without its x solve: 61 M warp instructions and 0.123 ms, against 94 M and 0.150 ms for one
-// column per thread with the (x, p) halves of a node packed; 8192 x 8192 with the deposit alone 0.395 ms
-// against 0.473, in one pass with both solves 0.512 against 0.632.
+// column per thread with the (x, p) halves of a node packed; 8192 x 8192 with the deposit alone 0.357 ms
+// against 0.473, in one pass with both solves 0.479 against 0.632 (0.395 and 0.512 while steps were not launched
+// ahead and lost weight was added cell by cell in FP64).
 //
 // What mattered beside the packing, in instructions of the row loop: no function call in it (the calling
 // convention cost moves and spills), no copy of the 32 accumulators between the common path and the restart
@@ -114,7 +115,8 @@ struct WalkWin {
 // Weight of a row's cells a (window columns ca ..) and b (cb ..) that the tile counts as lost, countA, countB: the
 // rows that are. Error-free sums of both columns in packed FP32 (the row's total to 2^-48), so that FP64, which
 // runs at a 64th of the rate, is left with one addition a row: with the cells converted and added one by one,
-// tiles beyond whose edge many rows land took 7000 cycles a source row (640 x 512 rotated by pi / 10: 240 us a step, 170 so).
+// tiles beyond whose edge many rows land took 7000 cycles a source row (640 x 512 rotated by pi / 10: 240 us a step, 170
+// so; the shorter code also helps meshes that lose nothing, 8192 x 8192 0.490 -> 0.479 ms).
 template <int N>
 __device__ __forceinline__ void lose_row(const WalkWin *W, const f2_t *acc, bool countA, int ca, bool countB, int cb,
                                          double &lost)
