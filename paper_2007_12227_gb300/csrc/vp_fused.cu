@@ -915,13 +915,14 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
     }
     __syncthreads();
 
-    // ---- window rows beyond the open momentum edge: lost weight of the own columns
-    if (W.WP0 < 0 || W.WP0 + W.WH > np)
-    for (int rr = 0; rr < W.WH; ++rr) {
-        const int grow = rr + W.WP0;
-        if (grow >= 0 && grow < np) continue;
+    // ---- guard rows beyond an open momentum edge that the tile owns: lost weight of the own columns. Where tiles are
+    // lower than the guard, other tiles' windows reach past the mesh too; what lands there is the owner's to count
+    const int edge = (P0 == 0 ? 1 : 0) | (P0 + TPe == np ? 2 : 0);
+    for (int k = 0; k < 2 * Gp; ++k) {   // the rows below the tile, then those above it
+        if (!(edge & (k < Gp ? 1 : 2))) continue;
+        const T *row = win + (size_t)(k < Gp ? k : TPe + k) * W.ws;
         const int c0 = full ? 0 : W.own_c0, c1 = full ? W.WW : W.own_c1;
-        for (int c = c0 + tid; c < c1; c += blockDim.x) lost += wraw(win + rr * W.ws + c);
+        for (int c = c0 + tid; c < c1; c += blockDim.x) lost += wraw(row + c);
     }
     if (full) {
         // fold the guard columns onto the period: [-G, 0) -> [nx - G, nx), [nx, nx + G) -> [0, G)

@@ -186,9 +186,10 @@ struct Walk32 {
 };
 
 // One row of a pair's rings into the window. Rows outside the window belong to other tiles: they are clamped
-// into the window's guard rows, which nobody reads (a predicate on a shared-memory reduction becomes a
-// branch around it), in their own columns (one common place for them all serialised the warp's additions: 3900
-// cycles a row where strong shear carries most rows outside). In a tile at an open edge they count as lost, and zeros are added in their place.
+// into the window's guard rows (a predicate on a shared-memory reduction becomes a branch around it), in their own
+// columns (one common place for them all serialised the warp's additions: 3900 cycles a row where strong shear carries
+// most rows outside). Guard rows are read only in a tile that owns an open edge, and on that edge's side: there the
+// rows beyond count as lost here, and zeros are added in their place.
 template <int N>
 __device__ __forceinline__ void leave_row(const Walk32 &K, const f2_t *acc, int off, int dBA, int cA, int cB, double &lost)
 {

@@ -1,0 +1,78 @@
+"""What a tile must not count.
+
+Lost weight: rows beyond the open momentum edge are counted by the tile that owns that edge and by no other, also
+where another tile's window reaches past the mesh (tiles, or a last row of tiles, lower than the window's guard
+rows) and where rows beyond the window are clamped into those guard rows.
+
+Bounds: weights as in the other oracle comparisons (FP64 1e-12 relative L-infinity, FP32 1e-5 relative L1 of one to
+three steps). The lost weight is a sum of the same deposits: in FP32 within 1e-5 of the whole mass; in FP64 the weights'
+bound over the steps' sums, 1e-10 of the loss itself."""
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle import oracle as O  # noqa: E402
+from paper_2007_12227_gb300 import inputs as I  # noqa: E402
+from paper_2007_12227_gb300 import vlasov as V  # noqa: E402
+
+PI = math.pi
+FP32_TOL, FP64_TOL = 1e-5, 1e-12
+T, B3 = I.BASIS_TENT, I.BASIS_CUBIC
+GAL, LUMP = I.PROJ_GALERKIN, I.PROJ_LUMPED
+AUTO, FUSED, XP = V.VP_KERNEL_AUTO, V.VP_KERNEL_FUSED, V.VP_KERNEL_FUSED_XPASS
+
+
+def run(wl, kernel, tile, steps):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    f = I.make_f0(wl)
+    if wl.precision == I.FP32:
+        f = f.astype(np.float32)
+    sim = V.Sim(wl.grid, wl.basis, wl.pusher, precision=wl.precision, projection=wl.projection, kernel=kernel,
+                tile_x=tile[0], tile_p=tile[1])
+    plan = sim.plan()
+    sim.set_f(f)
+    sim.step(steps)
+    got, mom = sim.get_f(), sim.moments()
+    sim.close()
+    st = O.State(wl.grid, wl.pusher, O.TENT if wl.basis == T else O.CUBIC,
+                 O.GALERKIN if wl.projection == GAL else O.LUMPED, f.astype(np.float64))
+    st.run(steps)
+    if wl.precision == I.FP64:
+        e = np.abs(got - st.w).max() / np.abs(st.w).max()
+        assert e <= FP64_TOL, f"rel Linf {e:.3e}"
+    else:
+        e = np.abs(got - st.w).sum() / np.abs(st.w).sum()
+        assert e <= FP32_TOL, f"rel L1 {e:.3e}"
+    area = wl.grid.hx * wl.grid.hp
+    return mom, st.lost[0] * area, f.astype(np.float64).sum() * area, plan
+
+
+# nx, np, precision, basis, projection, kernel, tile: a last row of tiles of 1 to 3 rows (FP32, four guard rows), tiles and
+# last rows of tiles lower than eight (FP64), whole-period and windowed tiles, several row segments, both x passes
+LOSSY = {
+    "fp32_last1": (400, 49, I.FP32, B3, GAL, AUTO, (0, 16)), "fp32_default121": (300, 121, I.FP32, B3, GAL, AUTO, (0, 0)),
+    "fp32_default75": (357, 75, I.FP32, B3, GAL, AUTO, (0, 0)), "fp32_lumped": (300, 73, I.FP32, B3, LUMP, AUTO, (0, 0)),
+    "fp32_tent": (300, 50, I.FP32, T, GAL, AUTO, (96, 16)), "fp32_full": (120, 50, I.FP32, B3, GAL, AUTO, (0, 24)),
+    "fp32_xpass": (500, 65, I.FP32, B3, GAL, XP, (96, 16)), "fp32_low": (300, 31, I.FP32, B3, GAL, FUSED, (64, 2)),
+    "fp64_tent128": (128, 128, I.FP64, T, GAL, AUTO, (0, 0)), "fp64_cubic128": (128, 128, I.FP64, B3, GAL, AUTO, (0, 0)),
+    "fp64_last2": (275, 66, I.FP64, B3, GAL, FUSED, (64, 64)), "fp64_last7": (400, 71, I.FP64, T, GAL, AUTO, (96, 32)),
+    "fp64_xpass": (301, 67, I.FP64, B3, GAL, AUTO, (0, 0)), "fp64_low": (200, 40, I.FP64, B3, LUMP, FUSED, (64, 3)),
+}
+
+
+@pytest.mark.parametrize("name", LOSSY)
+def test_lost_weight_is_counted_once(name):
+    nx, np_, prec, basis, proj, kernel, tile = LOSSY[name]
+    g = I.Grid(nx, np_, -PI, PI, -1.0, 1.0)
+    for pc in (0.8, -0.8):   # kicks of several rows across the upper and the lower edge
+        wl = I.Workload(name, g, I.Pusher(I.PUSH_KDK, I.POT_PENDULUM, 1.0, 1.0, 0.3), basis, prec, 2, "gaussian",
+                        dict(xc=1.0, pc=pc, sx=1.2, sp=0.15), projection=proj)
+        mom, lost, mass, _ = run(wl, kernel, tile, 2)
+        assert lost > 0.02 * mass, "the flow has to lose weight"
+        tol = 1e-10 * lost if prec == I.FP64 else FP32_TOL * mass
+        assert abs(mom["lost_mass"] - lost) <= tol, f"{name}: {mom['lost_mass']:.6f} for {lost:.6f} of {mass:.6f}"
