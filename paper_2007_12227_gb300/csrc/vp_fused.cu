@@ -533,10 +533,11 @@ __device__ __forceinline__ void solve_rows_f32(float *win, const WinGeom &W, flo
 
 // Rows of [ja, jb] from which the columns c0 .. c1 (unwrapped, up to nx of them) can reach the widened tile, by one
 // warp: the bounds of the tile's source rectangle for these columns alone. Called where the rectangle is much
-// taller than the tile: strong shear along p, or columns across the period of a force that is not periodic.
+// taller than the tile: strong shear along p, or columns across the period of a force that is not periodic. period: the
+// tile walks one whole period of columns, each for all its images.
 template <typename T>
 __device__ __forceinline__ int2 rows_of_columns(const FusedArgs<T> &A, int c0, int c1, int ja, int jb, int X0, int TXe, int P0,
-                                             int TPe, int D, int R, float Mf, float phif)
+                                             int TPe, int D, int R, float Mf, float phif, bool period)
 {
     const Geometry &g = A.g;
     const float SL = 0.05f;
@@ -567,7 +568,10 @@ __device__ __forceinline__ int2 rows_of_columns(const FusedArgs<T> &A, int c0, i
         const float vlo = (float)j + rb.y + vcl + tlo - SL, vhi = (float)j + rb.y + vch + thi + SL;
         const int ia = (int)floorf((float)(X0 - D - R) - rb.x - EU - (float)g.uc_max - SL);
         const int ib = (int)ceilf((float)(X0 + TXe + D - 1 + R) - rb.x + EU - (float)g.uc_min + SL);
-        if (vhi > acc_lo && vlo < acc_hi && (A.full_row || (c0 <= ib && c1 >= ia))) {
+        bool reach = A.full_row || (c0 <= ib && c1 >= ia);
+        if (period && !reach)   // an image of c0 in [ia, ib], or one of ia in [c0, c1]
+            reach = ib - ia + 1 >= g.nx || imod(c0 - ia, g.nx) <= ib - ia || imod(ia - c0, g.nx) <= c1 - c0;
+        if (vhi > acc_lo && vlo < acc_hi && reach) {
             lo = min(lo, j);
             hi = max(hi, j);
         }
@@ -667,7 +671,6 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
             s_win.own_c1 = full ? W.WW : W.own_c1;
             s_win.np = np;
             s_win.nx = nx;
-            s_win.full = full;
             s_win.edge = (P0 == 0 ? 1 : 0) | (P0 + TPe == np ? 2 : 0);
         }
     }
@@ -762,8 +765,18 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         ib = s_ib;
         ja = s_ja;
         jb = s_jb;
+        // Strong shear along x: the rows' source columns together span more than a period. Each column is then walked
+        // once, and its nodes land at their images in the window (a column that counted for one of its images alone
+        // left out the others: 28% of the weight of 640 x 512 turned by 1 rad). The period is centred on the tile,
+        // from an even column on (pairs in 8-byte loads)
+        if (!full && jb >= ja && (unsigned)ib - (unsigned)ia >= (unsigned)nx) {
+            ia = (X0 + (TXe - nx) / 2) & ~1;
+            ib = ia + nx - 1;
+        }
         if (A.tile_src && tid == 0) A.tile_src[tile] = make_int4(ia, ib, ja, jb);
     }
+    const bool period = !full && jb >= ja && ib - ia + 1 == nx;
+    if (tid == 0) s_win.wrap = full ? G : (period ? 0 : -1);
     double lost = 0.0;   // in the window's scaled units until the end of the tile
 
     // ---- the row table of the source rows into shared memory, when it fits: every node of a
@@ -829,7 +842,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         for (int wi = warp; wi < nwp; wi += nwarps) {
             const int c0 = ia2 + 64 * wi;
             int2 r = rows_of_columns<T>(A, c0, min(c0 + 63, ia2 + wsrc - 1), ja, jb, X0, TXe, P0, TPe, D, R, (float)M,
-                                        (float)phi);
+                                        (float)phi, period);
             if (r.x > r.y) r = make_int2(1, 0);
             if (lane == 0) s_rows[wi] = r;
         }

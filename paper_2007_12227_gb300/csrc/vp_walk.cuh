@@ -108,7 +108,8 @@ struct WalkWin {
     int WP0;                 // grid row of window row 0
     int own_c0, own_c1;      // the columns whose lost weight the tile counts
     int np, nx;
-    int full;                // the tile spans the whole period
+    int wrap;                // the tile walks a whole period of source columns: first window column of the images that
+                             // their nodes land at; else -1
     int edge;                // the tile owns the first (1), the last (2) mesh row: it counts the weight lost there
 };
 
@@ -138,15 +139,17 @@ __device__ __forceinline__ void lose_row(const WalkWin *W, const f2_t *acc, bool
     if (s.hi != 0.f || s.lo != 0.f) lost += s.value();
 }
 
-// Window column of a node's first tap, m, where it lies outside [0, WW - N]. In whole-period tiles it wraps (its
-// N cells then end in the right guard band at the latest, which is folded); in other tiles its cells belong to
-// other tiles or to the guard band, at least N wide, which nobody reads: it is moved into the band.
+// Window column of a node's first tap, m, where it lies outside [0, WW - N]. Where the tile walks a whole period of
+// source columns, the node lands at its image: in a whole-period tile (from the first own column on) the N cells end in
+// the right guard band at the latest, which is folded; a narrower window (from its first column on) holds one image
+// of a column at most. What is still outside belongs to other tiles or to the guard band, at least N wide, which
+// nobody reads: it is moved into the band.
 template <int N>
 __device__ __forceinline__ int fold_col(const WalkWin *W, int m)
 {
-    if (W->full) {
-        m = (m - W->G) % W->nx;
-        return W->G + (m < 0 ? m + W->nx : m);
+    if (W->wrap >= 0) {
+        m = (m - W->wrap) % W->nx;
+        return min(W->wrap + (m < 0 ? m + W->nx : m), W->WW - N);
     }
     return m < 0 ? 0 : W->WW - N;
 }

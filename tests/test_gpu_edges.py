@@ -1,8 +1,10 @@
-"""What a tile must not count.
+"""What a tile must not count and must not miss.
 
 Lost weight: rows beyond the open momentum edge are counted by the tile that owns that edge and by no other, also
 where another tile's window reaches past the mesh (tiles, or a last row of tiles, lower than the window's guard
 rows) and where rows beyond the window are clamped into those guard rows.
+
+Strong shear: where the source columns of a tile span more than a period, every node still lands once.
 
 Bounds: weights as in the other oracle comparisons (FP64 1e-12 relative L-infinity, FP32 1e-5 relative L1 of one to
 three steps). The lost weight is a sum of the same deposits: in FP32 within 1e-5 of the whole mass; in FP64 the weights'
@@ -76,3 +78,54 @@ def test_lost_weight_is_counted_once(name):
         assert lost > 0.02 * mass, "the flow has to lose weight"
         tol = 1e-10 * lost if prec == I.FP64 else FP32_TOL * mass
         assert abs(mom["lost_mass"] - lost) <= tol, f"{name}: {mom['lost_mass']:.6f} for {lost:.6f} of {mass:.6f}"
+
+
+def rot(nx, np_, angle):
+    return I.Grid(nx, np_, -4.0, 4.0, -4.0, 4.0), I.Pusher(I.PUSH_ROTATION, I.POT_HARMONIC, 1.0, 1.0, angle)
+
+
+def stream(nx, np_, dt):
+    return I.Grid(nx, np_, -PI, PI, -3.0, 3.0), I.Pusher(I.PUSH_KDK, I.POT_FREE, 1.0, 1.0, dt)
+
+
+def pend(nx, np_, dt):
+    return I.Grid(nx, np_, -PI, PI, -4.0, 4.0), I.Pusher(I.PUSH_KDK, I.POT_PENDULUM, 1.0, 1.0, dt)
+
+
+def fel(nx, np_, dt):
+    return I.Grid(nx, np_, 0.0, 2 * PI, -2.0, 2.0), I.Pusher(I.PUSH_FEL, I.POT_FREE, 1.0, 1.0, dt, 0.3, 0.0)
+
+
+SHEAR = {
+    "rot_fp64_255": (rot(255, 200, 1.0), I.FP64, B3, GAL, AUTO, (0, 0)),
+    "rot_fp64_256": (rot(256, 200, 1.3), I.FP64, B3, GAL, AUTO, (0, 0)),
+    "rot_fp64_lumped": (rot(200, 200, 1.0), I.FP64, B3, LUMP, AUTO, (0, 0)),
+    "rot_fp64_xpass": (rot(333, 150, 1.3), I.FP64, B3, GAL, AUTO, (0, 0)),
+    "rot_fp64_in_tile": (rot(300, 150, 1.2), I.FP64, B3, GAL, FUSED, (64, 24)),
+    "rot_fp32_640": (rot(640, 512, 1.0), I.FP32, B3, GAL, AUTO, (0, 0)),
+    "rot_fp32_odd": (rot(333, 200, 0.6), I.FP32, B3, GAL, AUTO, (0, 0)),
+    "rot_fp32_lumped": (rot(420, 330, 1.4), I.FP32, B3, LUMP, AUTO, (0, 0)),
+    "rot_fp32_tent": (rot(333, 200, 1.2), I.FP32, T, GAL, AUTO, (96, 24)),
+    "rot_fp32_xpass": (rot(400, 200, 1.1), I.FP32, B3, GAL, XP, (96, 32)),
+    "rot_fp32_tall": (rot(1300, 90, 1.2), I.FP32, B3, GAL, FUSED, (208, 64)),
+    "stream_fp32": (stream(320, 64, 1.0), I.FP32, B3, GAL, AUTO, (0, 0)),
+    "stream_fp32_far": (stream(321, 64, 9.0), I.FP32, B3, GAL, AUTO, (0, 0)),
+    "stream_fp64": (stream(320, 64, 1.0), I.FP64, B3, GAL, AUTO, (0, 0)),
+    "stream_fp64_tent": (stream(400, 50, 7.0), I.FP64, T, GAL, AUTO, (0, 0)),
+    "pend_fp32": (pend(300, 120, 2.5), I.FP32, B3, GAL, AUTO, (0, 0)),
+    "pend_fp64": (pend(300, 120, 2.5), I.FP64, B3, GAL, AUTO, (0, 0)),
+    "fel_fp32": (fel(300, 120, 2.0), I.FP32, B3, GAL, AUTO, (0, 0)),
+    "fel_fp64": (fel(300, 120, 2.0), I.FP64, B3, GAL, AUTO, (0, 0)),
+}
+
+
+@pytest.mark.parametrize("name", SHEAR)
+def test_every_node_lands_once_under_strong_shear(name):
+    (g, pu), prec, basis, proj, kernel, tile = SHEAR[name]
+    if pu.kind == I.PUSH_FEL:
+        wl = I.Workload(name, g, pu, basis, prec, 1, "fel_gaussian", dict(sp=0.8, eps=0.1), projection=proj)
+    else:
+        wl = I.Workload(name, g, pu, basis, prec, 1, "gaussian", dict(xc=0.5, pc=-0.3, sx=1.2, sp=1.0), projection=proj)
+    mom, lost, mass, plan = run(wl, kernel, tile, 1)
+    assert plan["kernel"] in (FUSED, XP), "a one-pass plan"
+    assert abs(mom["lost_mass"] - lost) <= (1e-10 * lost + 1e-12 * mass if prec == I.FP64 else FP32_TOL * mass)
