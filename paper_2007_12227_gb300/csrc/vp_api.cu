@@ -196,7 +196,9 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
         const int halo = P->galerkin && !P->xpass ? fused_halo(opts->precision) : 0;
         const int R = basis == VP_BASIS_TENT ? 1 : 2;
         const int G = P->G, Gp = P->Gp;
-        ftx = opts->tile_x ? opts->tile_x : (opts->precision == VP_FP64 ? 112 : (halo ? 208 : 240));
+        // FP32 by default: 256 columns with the halo and the guard (the x pass on a mesh that is no wider: 224)
+        const int width32 = halo ? 208 : (P->xpass && grid->nx <= 240 + 2 * G ? 224 : 240);
+        ftx = opts->tile_x ? opts->tile_x : (opts->precision == VP_FP64 ? 112 : width32);
         ftp = opts->tile_p ? opts->tile_p : 64;
         bool full = false;
         // whole-period tiles when the mesh is little wider than a windowed tile; by default only

@@ -1,0 +1,44 @@
+"""Default and asked-for plans on meshes near the planner's lines, against the oracle: the plan taken and its weights
+(FP64 <= 1e-12 relative L-infinity, FP32 <= 1e-5 relative L1, as in test_gpu_parity)."""
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle import oracle as O  # noqa: E402
+from paper_2007_12227_gb300 import inputs as I  # noqa: E402
+from paper_2007_12227_gb300 import vlasov as V  # noqa: E402
+
+PI = math.pi
+AUTO, FUSED, XP = V.VP_KERNEL_AUTO, V.VP_KERNEL_FUSED, V.VP_KERNEL_FUSED_XPASS
+
+
+def run(nx, np_, precision, kernel, tile=(0, 0), steps=5):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    wl = I.Workload("t", I.Grid(nx, np_, -PI, PI, -3.0, 3.0), I.Pusher(I.PUSH_KDK, I.POT_PENDULUM, 1.0, 1.0, 0.07),
+                    I.BASIS_CUBIC, precision, 0, "gaussian", dict(xc=0.0, pc=0.8, sx=0.5, sp=0.5))
+    f = I.make_f0(wl)
+    if precision == I.FP32:
+        f = f.astype(np.float32)
+    sim = V.Sim(wl.grid, wl.basis, wl.pusher, precision=precision, kernel=kernel, tile_x=tile[0], tile_p=tile[1])
+    plan = sim.plan()
+    sim.set_f(f)
+    sim.step(steps)
+    got = sim.get_f()
+    sim.close()
+    st = O.State(wl.grid, wl.pusher, O.CUBIC, O.GALERKIN, f.astype(np.float64))
+    st.run(steps)
+    if precision == I.FP64:
+        assert np.abs(got - st.w).max() <= 1e-12 * np.abs(st.w).max()
+    else:
+        assert np.abs(got - st.w).sum() <= 1e-5 * np.abs(st.w).sum()
+    return plan
+
+
+@pytest.mark.parametrize("nx", [241, 255, 256, 257])
+def test_separate_x_pass_fp32_on_a_mesh_little_wider_than_a_window(nx):
+    assert run(nx, 60, I.FP32, XP)["kernel"] == XP
