@@ -23,6 +23,8 @@ namespace {
 constexpr size_t kAlign = 256;
 constexpr int kDefaultHist = 4096;
 constexpr size_t kMaxSmem = 220 * 1024;
+constexpr int kGuardCols = 8;     // guard columns of a window: a multiple of 4, so that the x solve's rows start 16-byte aligned
+constexpr int kWholeSlack = 64;   // a mesh wider than a window by less than this takes whole-period tiles
 constexpr int kAutoXpassRow64 = 288;
 constexpr int kSlots = 2 * 152;   // CTAs of the step kernel the chip holds (two per SM)
 constexpr int kMoutLen = kMoutState + ST_NSTATE + 1;   // moments, step state, error flags
@@ -167,9 +169,15 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
     }
     // FP64 Galerkin by the planner's choice: rows longer than two windows take the separate x pass. An in-tile
     // solve needs 28 columns on both sides of a tile (1.5 times the tile's own columns at 112), all of them
-    // through the FP64 pipe; batches, which take the one-pass form only, hold FP32
+    // through the FP64 pipe; batches, which take the one-pass form only, hold FP32. A tile asked for by a width that
+    // covers the period, or nearly so, stays a whole-period tile: the pass has none, and without one such a mesh fell
+    // to the tiled kernel, or was refused where its tile is too large for that
+    const int beside = grid->nx - opts->tile_x;   // columns beside a tile of that width
+    const bool windowed = opts->tile_x == 0 ||
+                          (beside > 2 * kGuardCols && (grid->nx > kFusedMaxRow ||
+                                                       beside >= 2 * fused_halo(VP_FP64) + 2 * kGuardCols + kWholeSlack));
     const bool auto_x = kernel == VP_KERNEL_AUTO && opts->precision == VP_FP64 && P->galerkin && !P->rk4 &&
-                        !wide_rotation && grid->nx >= kAutoXpassRow64;
+                        !wide_rotation && grid->nx >= kAutoXpassRow64 && windowed;
     if (auto_x) {
         int xt = 0, xper = 0;
         xrow_shape(opts->precision, grid->nx, &xt, &xper);
@@ -183,7 +191,7 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
                         "the RK4 FEL step and the septic deposit run on the scatter kernel");
         kernel = VP_KERNEL_SCATTER;
     }
-    P->G = 8;   // a multiple of 4, so that the x solve's rows start 16-byte aligned
+    P->G = kGuardCols;
     // rows: FP32 rings drop rows outside the window in their common path, so four are enough there
     P->Gp = opts->precision == VP_FP64 ? 8 : 4;
     P->full_row = false;
@@ -205,7 +213,7 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
         // while the tile's source columns fit the two-CTA thread count (a default plan of more
         // threads runs one CTA per SM, and in a batch it would set that for every item)
         const bool full_fits = (grid->nx + 2 * R + 8 + 31) / 32 * 32 <= 320;
-        if (!P->xpass && grid->nx <= kFusedMaxRow && grid->nx < ftx + 2 * halo + 2 * G + 64 &&
+        if (!P->xpass && grid->nx <= kFusedMaxRow && grid->nx < ftx + 2 * halo + 2 * G + kWholeSlack &&
             (full_fits || opts->tile_x != 0 || grid->nx <= ftx + 2 * halo + 2 * G)) {
             full = true;
             ftx = grid->nx;
@@ -302,6 +310,7 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
                         "the fused kernel needs a mesh wider than its window (nx = %d)", grid->nx);
         } else {
             kernel = VP_KERNEL_TILED;
+            P->xpass = false;
         }
     }
     if (kernel == VP_KERNEL_TILED && wide_rotation) kernel = VP_KERNEL_SCATTER;

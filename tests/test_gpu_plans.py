@@ -42,3 +42,15 @@ def run(nx, np_, precision, kernel, tile=(0, 0), steps=5):
 @pytest.mark.parametrize("nx", [241, 255, 256, 257])
 def test_separate_x_pass_fp32_on_a_mesh_little_wider_than_a_window(nx):
     assert run(nx, 60, I.FP32, XP)["kernel"] == XP
+
+
+@pytest.mark.parametrize("nx,tile", [(300, (300, 128)), (357, (448, 128)), (300, (290, 0))])
+def test_fp64_tile_as_wide_as_the_mesh(nx, tile):
+    plan = run(nx, 130, I.FP64, AUTO, tile)
+    assert plan["kernel"] == FUSED and plan["full_row"] == 1
+
+
+@pytest.mark.parametrize("nx,tile,kernel", [(301, (0, 0), XP), (700, (0, 24), XP), (530, (400, 16), XP), (530, (530, 16), FUSED)])
+def test_fp64_default_x_pass_in_place(nx, tile, kernel):
+    """Odd rows, rows longer than a whole-period tile may be, tiles asked for (one leaves the pass's window no room)."""
+    assert run(nx, 75, I.FP64, AUTO, tile)["kernel"] == kernel

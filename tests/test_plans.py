@@ -23,3 +23,10 @@ def size(nx, np_, precision, kernel, tile_x=0, tile_p=0):
 def test_separate_x_pass_fp32_takes_meshes_little_wider_than_a_window(nx):
     """The default tile leaves the mesh wider than its window."""
     assert size(nx, 100, V.VP_FP32, V.VP_KERNEL_FUSED_XPASS) >= 2 * 4 * nx * 100
+
+
+@pytest.mark.parametrize("nx,tile", [(300, (300, 128)), (357, (448, 128)), (320, (480, 256)), (288, (400, 256))])
+def test_fp64_takes_tiles_as_wide_as_the_mesh(nx, tile):
+    """A whole-period tile, whatever the planner would choose by itself: no third mesh-sized buffer either."""
+    plain = size(nx, 130, V.VP_FP64, V.VP_KERNEL_FUSED, *tile)
+    assert abs(size(nx, 130, V.VP_FP64, V.VP_KERNEL_AUTO, *tile) - plain) < 8 * nx
