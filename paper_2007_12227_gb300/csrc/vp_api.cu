@@ -25,7 +25,7 @@ constexpr int kDefaultHist = 4096;
 constexpr size_t kMaxSmem = 220 * 1024;
 constexpr int kGuardCols = 8;     // guard columns of a window: a multiple of 4, so that the x solve's rows start 16-byte aligned
 constexpr int kWholeSlack = 64;   // a mesh wider than a window by less than this takes whole-period tiles
-constexpr int kAutoXpassRow64 = 288;
+constexpr int kAutoXpassRow64 = 176;
 constexpr int kSlots = 2 * 152;   // CTAs of the step kernel the chip holds (two per SM)
 constexpr int kMoutLen = kMoutState + ST_NSTATE + 1;   // moments, step state, error flags
 
@@ -167,9 +167,11 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
         P->xpass = true;
         kernel = VP_KERNEL_FUSED;
     }
-    // FP64 Galerkin by the planner's choice: rows longer than two windows take the separate x pass. An in-tile
+    // FP64 Galerkin by the planner's choice: rows of 176 nodes and more take the separate x pass. An in-tile
     // solve needs 28 columns on both sides of a tile (1.5 times the tile's own columns at 112), all of them
-    // through the FP64 pipe; batches, which take the one-pass form only, hold FP32. A tile asked for by a width that
+    // through the FP64 pipe, or whole-period tiles, which are few and low (a step of 233 x 828: 98 us with the pass,
+    // 176 without; of 252 x 580 80 and 164; of 190 x 154 61 and 65; of 157 x 97 61 and 59). Batches, which take the
+    // one-pass form only, hold FP32. A tile asked for by a width that
     // covers the period, or nearly so, stays a whole-period tile: the pass has none, and without one such a mesh fell
     // to the tiled kernel, or was refused where its tile is too large for that
     const int beside = grid->nx - opts->tile_x;   // columns beside a tile of that width

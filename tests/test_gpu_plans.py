@@ -54,3 +54,8 @@ def test_fp64_tile_as_wide_as_the_mesh(nx, tile):
 def test_fp64_default_x_pass_in_place(nx, tile, kernel):
     """Odd rows, rows longer than a whole-period tile may be, tiles asked for (one leaves the pass's window no room)."""
     assert run(nx, 75, I.FP64, AUTO, tile)["kernel"] == kernel
+
+
+@pytest.mark.parametrize("nx,np_", [(175, 90), (176, 90), (201, 300), (233, 828), (287, 61)])
+def test_fp64_rows_either_side_of_the_x_pass_line(nx, np_):
+    assert run(nx, np_, I.FP64, AUTO, steps=3)["kernel"] == (XP if nx >= 176 else FUSED)
