@@ -708,7 +708,7 @@ struct StateBlock {
 };
 struct ZeroRanges {
     unsigned *p[5];
-    unsigned n[5];   // 4-byte words
+    size_t n[5];   // 4-byte words (a field history alone may hold 2^33 of them)
 };
 __global__ void reset_kernel(double *dst, StateBlock b, ZeroRanges z)
 {
@@ -716,7 +716,8 @@ __global__ void reset_kernel(double *dst, StateBlock b, ZeroRanges z)
         for (int k = threadIdx.x; k < ST_NSTATE; k += blockDim.x) dst[k] = b.v[k];
 #pragma unroll
     for (int q = 0; q < 5; ++q)
-        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < z.n[q]; k += gridDim.x * blockDim.x) z.p[q][k] = 0u;
+        for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < z.n[q]; k += (size_t)gridDim.x * blockDim.x)
+            z.p[q][k] = 0u;
 }
 
 vp_status reset_state(vp_sim *s, const void *w)
@@ -732,7 +733,7 @@ vp_status reset_state(vp_sim *s, const void *w)
     memset(&z, 0, sizeof(z));
     auto zero = [&](int q, size_t off, size_t bytes) {
         z.p[q] = s->ptr<unsigned>(off);
-        z.n[q] = (unsigned)(bytes / 4);
+        z.n[q] = bytes / 4;
     };
     zero(0, P.L.lost, (size_t)P.nlost * sizeof(double));
     zero(1, P.L.err, sizeof(unsigned));

@@ -59,3 +59,27 @@ def test_fp64_default_x_pass_in_place(nx, tile, kernel):
 @pytest.mark.parametrize("nx,np_", [(175, 90), (176, 90), (201, 300), (233, 828), (287, 61)])
 def test_fp64_rows_either_side_of_the_x_pass_line(nx, np_):
     assert run(nx, np_, I.FP64, AUTO, steps=3)["kernel"] == (XP if nx >= 176 else FUSED)
+
+
+def test_reset_zeroes_a_field_history_of_four_billion_words():
+    """set_f zeroes the history ring: 2^32 - 4000 words here, more than a 32-bit count of the zeroing threads' steps holds."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    cap = (1 << 30) - 1000
+    g = I.Grid(64, 32, 0.0, 2 * PI, -0.5, 0.5)
+    pu = I.Pusher(I.PUSH_FEL, I.POT_FREE, 1.0, 1.0, 0.05, 0.3, 0.0)
+    if torch.cuda.mem_get_info()[0] < 18 * cap:
+        pytest.skip("needs 18 GB")
+    # the workspace takes this freed block, so that its history is not zero to begin with
+    block = torch.empty(16 * cap + (1 << 20), dtype=torch.uint8, device="cuda").fill_(255)
+    del block
+    sim = V.Sim(g, I.BASIS_CUBIC, pu, precision=V.VP_FP32, history_cap=cap)
+    sim.set_f(np.ones((32, 64), dtype=np.float32))
+    sim.sync()
+    size = sim.workspace.numel()
+    margin = (size - 16 * cap + 255) // 256 * 256   # what else the workspace holds, before or behind the history
+    words = sim.workspace[margin: 16 * cap // 256 * 256].view(torch.int64)
+    assert not any(bool(c.any()) for c in words.split(1 << 28))
+    sim.close()
+    del sim, words
+    torch.cuda.empty_cache()
