@@ -940,11 +940,22 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
     if (full) {
         // fold the guard columns onto the period: [-G, 0) -> [nx - G, nx), [nx, nx + G) -> [0, G)
         __syncthreads();
-        for (int k = tid; k < TPe * G; k += blockDim.x) {
-            const int rr = k / G + Gp, c = k - (k / G) * G;
-            T *row = win + (size_t)rr * W.ws;
-            wfold(row + nx + c, row + c);
-            wfold(row + G + c, row + G + nx + c);
+        if (nx >= G) {
+            for (int k = tid; k < TPe * G; k += blockDim.x) {
+                const int rr = k / G + Gp, c = k - (k / G) * G;
+                T *row = win + (size_t)rr * W.ws;
+                wfold(row + nx + c, row + c);
+                wfold(row + G + c, row + G + nx + c);
+            }
+        } else {
+            // a band longer than the period: several of its columns have the same image
+            for (int rr = tid; rr < TPe; rr += blockDim.x) {
+                T *row = win + (size_t)(rr + Gp) * W.ws;
+                for (int c = 0; c < G; ++c) {
+                    wfold(row + G + imod(c - G, nx), row + c);
+                    wfold(row + G + c % nx, row + G + nx + c);
+                }
+            }
         }
     }
     __syncthreads();

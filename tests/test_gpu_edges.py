@@ -129,3 +129,14 @@ def test_every_node_lands_once_under_strong_shear(name):
     mom, lost, mass, plan = run(wl, kernel, tile, 1)
     assert plan["kernel"] in (FUSED, XP), "a one-pass plan"
     assert abs(mom["lost_mass"] - lost) <= (1e-10 * lost + 1e-12 * mass if prec == I.FP64 else FP32_TOL * mass)
+
+
+@pytest.mark.parametrize("prec", [I.FP32, I.FP64], ids=["fp32", "fp64"])
+@pytest.mark.parametrize("basis", [T, B3], ids=["tent", "cubic"])
+@pytest.mark.parametrize("nx", [4, 5, 7, 8])
+def test_meshes_narrower_than_the_guard_band(nx, basis, prec):
+    """Nodes that land several periods' worth of columns away, in guard columns of which some share their image."""
+    for dt in (1.0, 3.0, 4.3):
+        g, pu = I.Grid(nx, 40, -PI, PI, -3.0, 3.0), I.Pusher(I.PUSH_KDK, I.POT_PENDULUM, 1.0, 1.0, dt)
+        wl = I.Workload("t", g, pu, basis, prec, 1, "gaussian", dict(xc=0.5, pc=-0.3, sx=1.2, sp=1.0), projection=GAL)
+        run(wl, AUTO, (0, 0), 1)
