@@ -563,7 +563,8 @@ vp_status fel_bunching(vp_sim *s, const void *w, int init)
     VP_CUDA(s, launch_fel_partials<T>(static_cast<const T *>(w), P.g.nx, P.g.np,
                                       s->ptr<double2>(P.L.csx), part, s->stream));
     VP_CUDA(s, launch_fel_finalize(part, fel_partial_blocks(P.g.nx, P.g.np), s->ptr<double>(P.L.state),
-                                   s->ptr<double>(P.L.hist), P.hist_cap, P.g.dt, init, s->stream));
+                                   s->ptr<double>(P.L.hist), P.hist_cap, P.g.dt, init, P.kernel == VP_KERNEL_TILED,
+                                   s->stream));
     return VP_OK;
 }
 
@@ -578,7 +579,7 @@ vp_status fel_space_charge(vp_sim *s, const void *st)
                                    rt, rt + P.g.np, P.state_s ? s->ptr<double>(P.L.sigma) : nullptr, part,
                                    s->stream));
     VP_CUDA(s, launch_fel_kick(part, fel_partial_blocks(P.g.nx, P.g.np), s->ptr<double>(P.L.state),
-                               P.g.sigma2, s->stream));
+                               P.g.sigma2, P.kernel == VP_KERNEL_TILED, s->stream));
     return VP_OK;
 }
 
@@ -686,7 +687,7 @@ vp_status do_steps(vp_sim *s, int n, cudaEvent_t *ev = nullptr)
         if (P.fel) {
             if (P.kernel != VP_KERNEL_FUSED)
                 VP_CUDA(s, launch_fel_finalize(part, nparts, state, s->ptr<double>(P.L.hist), P.hist_cap,
-                                               P.g.dt, 0, s->stream, P.rk4 ? 1 : 0));
+                                               P.g.dt, 0, P.kernel == VP_KERNEL_TILED, s->stream, P.rk4 ? 1 : 0));
             if (P.g.sigma2 != 0.0 && !P.rk4) {
                 const vp_status sc = fel_space_charge<T>(s, dst);
                 if (sc != VP_OK) return sc;

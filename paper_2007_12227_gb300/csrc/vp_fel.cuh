@@ -15,11 +15,18 @@ namespace vp {
 constexpr int kFinThreads = 256;
 static_assert(kFinSmem == 3 * kFinThreads * sizeof(double), "scratch of fel_finalize_core");
 
-// Amplitude and phase of the kick's sine term, alpha = -Im K, beta = Re K. They only bound the tiles' source
-// windows, with a slack of hundredths of a cell: FP32 (relative error 1e-6 at most, the amplitude rounded up) instead
-// of FP64 hypot and atan2 on the one thread that ends the step.
-__device__ __forceinline__ void store_kick_bounds(double *state)
+// Amplitude and phase of the kick's sine term, alpha = -Im K, beta = Re K: they bound the tiles' source windows, no more.
+// The one-pass kernel bounds them in FP32 with a slack of 1e-4 of the amplitude, so FP32 (relative error 1e-6 at most,
+// the amplitude rounded up) serves it; FP64 hypot and atan2 on the one thread that ends the step cost 1 to 2% of it (20
+// steps of 4096 x 2048 2111 us for 2087). The tiled kernel bounds them in FP64 (exact) with a slack of 0.02 cells, less than
+// an FP32 phase is off for kicks of more than some 28000 cells.
+__device__ __forceinline__ void store_kick_bounds(double *state, bool exact)
 {
+    if (exact) {
+        state[ST_M] = hypot(state[ST_K_RE], state[ST_K_IM]);
+        state[ST_PHI] = atan2(state[ST_K_RE], -state[ST_K_IM]);
+        return;
+    }
     const float re = (float)state[ST_K_RE], im = (float)state[ST_K_IM];
     state[ST_M] = (double)(hypotf(re, im) * 1.000001f);
     state[ST_PHI] = (double)atan2f(re, -im);
@@ -32,7 +39,7 @@ __device__ __forceinline__ void store_kick_bounds(double *state)
 // memory. Partials are read through L2 (other CTAs of the same launch may have written them).
 __device__ __forceinline__ void fel_finalize_core(const double *part, int nparts, double *state,
                                                   double *hist, int hist_cap, double dt, int init,
-                                                  int rk4, double *s)
+                                                  int rk4, bool exact_bounds, double *s)
 {
     const int t = threadIdx.x, nt = blockDim.x;
     for (int v = t; v < kFinThreads; v += nt) {
@@ -64,7 +71,7 @@ __device__ __forceinline__ void fel_finalize_core(const double *part, int nparts
         // kick amplitude K = A^{1/2} (space charge adds i sigma2 <e^{-i theta~}> afterwards)
         state[ST_K_RE] = state[ST_AH_RE];
         state[ST_K_IM] = state[ST_AH_IM];
-        store_kick_bounds(state);
+        store_kick_bounds(state, exact_bounds);
         return;
     }
     // DKD: A^{n+1} = A^{n+1/2} + h/2 b^{n+1}; RK4: the stages left A^{n+1} in ST_AH
@@ -77,7 +84,7 @@ __device__ __forceinline__ void fel_finalize_core(const double *part, int nparts
     state[ST_K_RE] = state[ST_AH_RE];
     state[ST_K_IM] = state[ST_AH_IM];
     // sine-term weights of the next push: alpha = -Im K, beta = Re K
-    store_kick_bounds(state);
+    store_kick_bounds(state, exact_bounds);
     const long step = (long)state[ST_STEP];
     if (hist && hist_cap > 0) {
         const long slot = step % hist_cap;

@@ -1091,7 +1091,7 @@ __device__ __forceinline__ bool finish_step(const FusedArgs<T> &A, unsigned char
     __threadfence();
     double *state = const_cast<double *>(A.state);
     if (A.fel_partials) {
-        fel_finalize_core(A.tile_part, A.ntx * A.ntp, state, A.hist, A.hist_cap, A.g.dt, 0, 0,
+        fel_finalize_core(A.tile_part, A.ntx * A.ntp, state, A.hist, A.hist_cap, A.g.dt, 0, 0, false,
                           reinterpret_cast<double *>(smem_raw));
     } else if (threadIdx.x == 0) {
         const double st = state[ST_STEP] + 1.0;

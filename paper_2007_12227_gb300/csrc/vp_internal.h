@@ -278,7 +278,8 @@ int fel_partial_blocks(int nx, int np);
 template <typename T>
 cudaError_t launch_fel_tilde(const T *state, int nx, int np, const double2 *csx, const double *rc,
                              const double *rs, const double *sig, double *part, cudaStream_t s);
-cudaError_t launch_fel_kick(const double *part, int nparts, double *state, double sigma2,
+// exact_bounds: store_kick_bounds in FP64 (the tiled kernel reads them so)
+cudaError_t launch_fel_kick(const double *part, int nparts, double *state, double sigma2, bool exact_bounds,
                             cudaStream_t s);
 // FEL RK4: the stage reductions and amplitudes (rt: cos and sin of the half drift per row; part:
 // 5 rk4_stage_blocks doubles), and the deposit at the RK4 end points into a zeroed destination
@@ -291,7 +292,7 @@ cudaError_t launch_rk4_deposit(const T *src, T *dst, const Geometry &g, const do
                                const double *state, double *lost_acc, cudaStream_t s);
 // init: first bunching after vp_set_f; rk4: A^{n+1} is the RK4 value left in ST_AH
 cudaError_t launch_fel_finalize(const double *part, int nparts, double *state, double *hist,
-                                int hist_cap, double dt, int init, cudaStream_t s, int rk4 = 0);
+                                int hist_cap, double dt, int init, bool exact_bounds, cudaStream_t s, int rk4 = 0);
 cudaError_t launch_count_step(double *state, double dt, cudaStream_t s);
 
 // ln: the table of ln of FP32 weights that build_ln_table writes (kLnTableBytes)

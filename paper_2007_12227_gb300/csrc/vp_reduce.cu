@@ -105,7 +105,8 @@ __global__ void fel_tilde_kernel(const T *__restrict__ st, int nx, int np, const
 }
 
 // K = A^{n+1/2} + i sigma2 bt, bt = <e^{-i theta~}> from the tilde partial sums (one block)
-__global__ void fel_kick_kernel(const double *__restrict__ part, int nparts, double *state, double sigma2)
+__global__ void fel_kick_kernel(const double *__restrict__ part, int nparts, double *state, double sigma2,
+                                bool exact_bounds)
 {
     __shared__ double s[3][kRedThreads];
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
@@ -128,21 +129,15 @@ __global__ void fel_kick_kernel(const double *__restrict__ part, int nparts, dou
     const double kr = state[ST_AH_RE] - sigma2 * bt_im, ki = state[ST_AH_IM] + sigma2 * bt_re;
     state[ST_K_RE] = kr;
     state[ST_K_IM] = ki;
-    store_kick_bounds(state);
+    store_kick_bounds(state, exact_bounds);
 }
 
 // FEL field update from per-block partial sums (run by one block of kFinThreads threads)
-__device__ void fel_finalize_block(const double *__restrict__ part, int nparts, double *state,
-                                   double *hist, int hist_cap, double dt, int init, int rk4 = 0)
+__global__ void fel_finalize_kernel(const double *__restrict__ part, int nparts, double *state, double *hist,
+                                    int hist_cap, double dt, int init, int rk4, bool exact_bounds)
 {
     __shared__ double s[3 * kFinThreads];
-    fel_finalize_core(part, nparts, state, hist, hist_cap, dt, init, rk4, s);
-}
-
-__global__ void fel_finalize_kernel(const double *__restrict__ part, int nparts, double *state,
-                                    double *hist, int hist_cap, double dt, int init, int rk4)
-{
-    fel_finalize_block(part, nparts, state, hist, hist_cap, dt, init, rk4);
+    fel_finalize_core(part, nparts, state, hist, hist_cap, dt, init, rk4, exact_bounds, s);
 }
 
 // plain step counter for non-FEL sims
@@ -382,9 +377,10 @@ template cudaError_t launch_fel_tilde<float>(const float *, int, int, const doub
 template cudaError_t launch_fel_tilde<double>(const double *, int, int, const double2 *, const double *,
                                               const double *, const double *, double *, cudaStream_t);
 
-cudaError_t launch_fel_kick(const double *part, int nparts, double *state, double sigma2, cudaStream_t s)
+cudaError_t launch_fel_kick(const double *part, int nparts, double *state, double sigma2, bool exact_bounds,
+                            cudaStream_t s)
 {
-    fel_kick_kernel<<<1, kRedThreads, 0, s>>>(part, nparts, state, sigma2);
+    fel_kick_kernel<<<1, kRedThreads, 0, s>>>(part, nparts, state, sigma2, exact_bounds);
     return cudaGetLastError();
 }
 
@@ -398,9 +394,9 @@ cudaError_t launch_fel_partials(const T *w, int nx, int np, const double2 *csx, 
 }
 
 cudaError_t launch_fel_finalize(const double *part, int nparts, double *state, double *hist,
-                                int hist_cap, double dt, int init, cudaStream_t s, int rk4)
+                                int hist_cap, double dt, int init, bool exact_bounds, cudaStream_t s, int rk4)
 {
-    fel_finalize_kernel<<<1, kRedThreads, 0, s>>>(part, nparts, state, hist, hist_cap, dt, init, rk4);
+    fel_finalize_kernel<<<1, kRedThreads, 0, s>>>(part, nparts, state, hist, hist_cap, dt, init, rk4, exact_bounds);
     return cudaGetLastError();
 }
 
