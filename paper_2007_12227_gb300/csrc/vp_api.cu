@@ -26,7 +26,7 @@ constexpr size_t kMaxSmem = 220 * 1024;
 constexpr int kGuardCols = 8;     // guard columns of a window: a multiple of 4, so that the x solve's rows start 16-byte aligned
 constexpr int kWholeSlack = 64;   // a mesh wider than a window by less than this takes whole-period tiles
 constexpr int kAutoXpassRow64 = 176;
-constexpr int kSlots = 2 * 152;   // CTAs of the step kernel the chip holds (two per SM)
+constexpr int kSlots = 2 * 152;   // CTAs of the step kernel the chip holds: two on each of its 152 SMs (wide tiles: one)
 constexpr int kMoutLen = kMoutState + ST_NSTATE + 1;   // moments, step state, error flags
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -258,21 +258,22 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
         const bool wide = wsrc > 320;   // one CTA per SM
         const size_t cap = wide ? (size_t)200 * 1024 : (size_t)112 * 1024;
         if (opts->tile_p == 0 && !pick64) {
+            const int slots = wide ? kSlots / 2 : kSlots;
             const int ntx = (grid->nx + ftx - 1) / ftx;
             auto tiles = [&](int h) { return (long)ntx * ((grid->np + h - 1) / h); };
-            if (tiles(ftp) <= kSlots) {
+            if (tiles(ftp) <= slots) {
                 // a mesh that does not fill the chip with such tiles: as low as gives every slot one (a tile's time
                 // is a fixed part of some 30 rows' worth plus its rows: 357 x 300 FP32 takes 37 us a step with 64
                 // rows, 22.8 with 24, 18.7 with 16; but in a batch, where other simulations fill the chip, low tiles
                 // only add the fixed part: 40 mixed ones take 132, 117 and 140 us)
                 const int least = opts->precision == VP_FP64 ? 4 : 24;   // FP64 here: whole-period tiles, not in batches
-                const int per_col = std::max(1, kSlots / ntx), h = (grid->np + per_col - 1) / per_col;
+                const int per_col = std::max(1, slots / ntx), h = (grid->np + per_col - 1) / per_col;
                 ftp = std::min(ftp, std::max(least, (h + 3) / 4 * 4));
             } else {
                 // a last wave of less than 0.4 of the slots costs nearly a whole one: lower tiles fill it (2048 x 2048
                 // FP32: 64 rows, 1.05 waves, 59.8 us a step; 48 rows, 1.41 waves, 49.5 us)
                 for (int h = ftp; h >= 40 && h <= 64; h -= 4) {
-                    const double waves = (double)tiles(h) / kSlots, last = waves - floor(waves);
+                    const double waves = (double)tiles(h) / slots, last = waves - floor(waves);
                     if (waves > 8.0 || last == 0.0 || last >= 0.4) {
                         ftp = h;
                         break;

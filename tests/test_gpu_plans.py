@@ -83,3 +83,10 @@ def test_reset_zeroes_a_field_history_of_four_billion_words():
     sim.close()
     del sim, words
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("nx,np_,precision,tile_x", [(709, 991, I.FP64, 384), (1500, 700, I.FP32, 448)])
+def test_wide_tiles_are_planned_at_one_block_an_sm(nx, np_, precision, tile_x):
+    """The default height gives every SM one such tile: fewer than 152 tiles, and more than half of that."""
+    plan = run(nx, np_, precision, FUSED, (tile_x, 0), steps=2)
+    assert 76 < plan["ntiles_x"] * plan["ntiles_p"] <= 152
