@@ -500,8 +500,6 @@ FusedArgs<T> fused_args(vp_sim *s, const void *src, void *dst)
     a.dst = static_cast<T *>(dst);
     a.col = s->ptr<ColEntry<T>>(P.L.col);
     a.row = s->ptr<RowEntry<T>>(P.L.row);
-    a.rowb = s->ptr<RowBound>(P.L.rowb);
-    a.vcb = s->ptr<double>(P.L.vcb);
     a.rowbf = s->ptr<float4>(P.L.rowbf);
     a.vcbf = s->ptr<float2>(P.L.vcbf);
     a.state = s->ptr<double>(P.L.state);

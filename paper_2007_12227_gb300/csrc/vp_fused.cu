@@ -126,49 +126,49 @@ struct WinGeom {
     int WW, WH, ws;      // window width, height, row stride (elements)
     int WX0, WP0;        // grid column (unwrapped) and row of window cell (0, 0)
     int own_c0, own_c1;  // the tile's own columns, window coordinates [c0, c1)
-    int np, nx, G;
+    int np, nx;
     bool full;           // the tile spans the whole period
 };
 
-// Lambda_x^{-1} (T x = row, T = tridiag(1/6, 2/3, 1/6)) of one row of length L held in
-// shared memory, by one warp. Returns each lane's elements base .. base + per - 1 in v.
-// cyclic: the row is one whole period; else the row is padded by the halo on both
-// sides and the recurrences start from zero at its ends (truncation |z|^halo).
+constexpr double kXScale64 = -6.0 * -0.26794919243112270647;   // -6 z, after the two recursions
 // padded staging layout of a row: element c at c + c / 8, so that lanes reading
 // contiguous chunks of 8 hit distinct shared-memory banks
 __device__ __forceinline__ int padc(int c) { return c + (c >> 3); }
 
-template <typename T, int kXMax>
-__device__ void solve_row_x(const T *row, int L, bool cyclic, int lane, T *v, int &per, int &base,
-                            bool padded, T sh, T sl)
+// FP64 Lambda_x^{-1} (T x = row, T = tridiag(1/6, 2/3, 1/6)) of one row of length L held in
+// shared memory, by one warp. Returns each lane's elements base .. base + per - 1 in v.
+// cyclic: the row is one whole period; else the row is padded by the halo on both
+// sides and the recurrences start from zero at its ends (truncation |z|^halo).
+template <int kXMax>
+__device__ void solve_row_x(const double *row, int L, bool cyclic, int lane, double *v, int &per, int &base, bool padded)
 {
     per = (L + 31) / 32;
     base = lane * per;
-    const T z = (T)-0.26794919243112270647;
+    const double z = -0.26794919243112270647;
 #pragma unroll
     for (int k = 0; k < kXMax; ++k)
-        v[k] = (k < per && base + k < L) ? row[padded ? padc(base + k) : base + k] : T(0);
-    const T zper = zpow<T>(per);
+        v[k] = (k < per && base + k < L) ? row[padded ? padc(base + k) : base + k] : 0.0;
+    const double zper = zpow<double>(per);
     // causal y_i = x_i + z y_{i-1}: lane-local sweep, then carries by a warp scan
-    T y = T(0);
+    double y = 0.0;
 #pragma unroll
     for (int k = 0; k < kXMax; ++k)
         if (k < per) {
             y = v[k] + z * y;
             v[k] = y;
         }
-    T endv = y;
-    T zp = zper;
+    double endv = y;
+    double zp = zper;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-        const T o = __shfl_up_sync(0xffffffffu, endv, off);
+        const double o = __shfl_up_sync(0xffffffffu, endv, off);
         if (lane >= off) endv += zp * o;
         zp *= zp;
     }
-    T carry = __shfl_up_sync(0xffffffffu, endv, 1);
-    if (lane == 0) carry = T(0);
+    double carry = __shfl_up_sync(0xffffffffu, endv, 1);
+    if (lane == 0) carry = 0.0;
     {
-        T zk = z;
+        double zk = z;
 #pragma unroll
         for (int k = 0; k < kXMax; ++k)
             if (k < per) {
@@ -179,13 +179,13 @@ __device__ void solve_row_x(const T *row, int L, bool cyclic, int lane, T *v, in
     if (cyclic) {
         // y_{-1} = y_{L-1}: with E the zero-start value at L-1, y_{-1} = E / (1 - z^L)
         const int ll = (L - 1) / per, kl = (L - 1) - ll * per;
-        T mine = T(0);
+        double mine = 0.0;
 #pragma unroll
         for (int k = 0; k < kXMax; ++k)
             if (k == kl) mine = v[k];
-        const T E = __shfl_sync(0xffffffffu, mine, ll);
-        const T yprev = E / (T(1) - zpow<T>(L));
-        T zk = zpow<T>(base + 1);
+        const double E = __shfl_sync(0xffffffffu, mine, ll);
+        const double yprev = E / (1.0 - zpow<double>(L));
+        double zk = zpow<double>(base + 1);
 #pragma unroll
         for (int k = 0; k < kXMax; ++k)
             if (k < per) {
@@ -196,25 +196,25 @@ __device__ void solve_row_x(const T *row, int L, bool cyclic, int lane, T *v, in
     // anticausal u_i = y_i + z u_{i+1}
     int last = per - 1;
     if (base + last >= L) last = L - 1 - base;   // may be negative for idle lanes
-    T u = T(0);
+    double u = 0.0;
 #pragma unroll
     for (int k = kXMax - 1; k >= 0; --k)
         if (k <= last) {
             u = v[k] + z * u;
             v[k] = u;
         }
-    T startv = u;
+    double startv = u;
     zp = zper;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-        const T o = __shfl_down_sync(0xffffffffu, startv, off);
+        const double o = __shfl_down_sync(0xffffffffu, startv, off);
         if (lane + off < 32) startv += zp * o;
         zp *= zp;
     }
-    T carry2 = __shfl_down_sync(0xffffffffu, startv, 1);
-    if (lane == 31) carry2 = T(0);
+    double carry2 = __shfl_down_sync(0xffffffffu, startv, 1);
+    if (lane == 31) carry2 = 0.0;
     {
-        T zk = z;
+        double zk = z;
 #pragma unroll
         for (int k = kXMax - 1; k >= 0; --k)
             if (k <= last) {
@@ -224,16 +224,15 @@ __device__ void solve_row_x(const T *row, int L, bool cyclic, int lane, T *v, in
     }
     if (cyclic) {
         // u_L = u_0: with S the zero-end value at 0, u_L = S / (1 - z^L)
-        const T S = __shfl_sync(0xffffffffu, v[0], 0);
-        const T unext = S / (T(1) - zpow<T>(L));
+        const double S = __shfl_sync(0xffffffffu, v[0], 0);
+        const double unext = S / (1.0 - zpow<double>(L));
         // element i gets z^{L - i} u_L
 #pragma unroll
         for (int k = 0; k < kXMax; ++k)
-            if (k <= last) v[k] += zpow<T>(L - (base + k)) * unext;
+            if (k <= last) v[k] += zpow<double>(L - (base + k)) * unext;
     }
-    // the scale -6z; in FP32 the unit-DC-gain scale of the step as a float pair sh + sl
 #pragma unroll
-    for (int k = 0; k < kXMax; ++k) v[k] = sizeof(T) == 4 ? v[k] * sh + v[k] * sl : v[k] * sh;
+    for (int k = 0; k < kXMax; ++k) v[k] *= kXScale64;
 }
 
 // z^n for the pole z = sqrt(3) - 2, at compile time
@@ -358,104 +357,48 @@ __device__ __forceinline__ void store_window_rows(const T *win, const WinGeom &W
     }
 }
 
-// Lambda_x solve of the tile's window rows (one warp per row) and the tile store.
-template <typename T, int KX>
-__device__ __forceinline__ void gal_rows(T *win, const WinGeom &W, T *dst, int L, bool full, int D,
-                                         int G, int Gp, int TXe, int TPe, int P0, int X0, int nx,
-                                         bool want_part, int warp, int nwarps, int lane, bool &bad,
-                                         T *stage_all, int stage_len, T sh, T sl, T iq, float &om)
+// FP64: Lambda_x solve of the tile's window rows (one warp per row) and the tile store.
+template <int KX>
+__device__ __forceinline__ void solve_rows_f64(double *win, const WinGeom &W, double *dst, int L, bool full, int D, int G,
+                                               int Gp, int TXe, int TPe, int P0, int X0, int nx, bool want_part, int warp,
+                                               int nwarps, int lane, bool &bad, double *stage_all, int stage_len)
 {
     // per-warp padded copy of the row (conflict-free reads of contiguous chunks)
     const int plen = padc(L) + 8;
-    const bool use_stage = stage_all != nullptr && (size_t)nwarps * plen <= (size_t)stage_len;
-    T *stage = use_stage ? stage_all + (size_t)warp * plen : nullptr;
+    const bool use_stage = (size_t)nwarps * plen <= (size_t)stage_len;
+    double *stage = stage_all + (size_t)warp * plen;
     for (int rr = warp; rr < TPe; rr += nwarps) {
-        T *row = win + (size_t)(rr + Gp) * W.ws + G;
-        T *dst_row = dst + (size_t)(P0 + rr) * nx + X0 - D;
-        T v[KX];
+        double *row = win + (size_t)(rr + Gp) * W.ws + G;
+        double *dst_row = dst + (size_t)(P0 + rr) * nx + X0 - D;
+        double v[KX];
         int per, base;
         const bool exact = !full && L == 32 * KX;
-        // FP32 rows of 32 KX cells starting 16-byte aligned: each lane reads its chunk of
-        // fixed-point cells with vector loads, without a staging copy
-        const bool direct = sizeof(T) == 4 && exact && KX % 4 == 0 &&
-                            ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
-        if (direct) {
-            const int4 *r4 = reinterpret_cast<const int4 *>(row + lane * KX);
-#pragma unroll
-            for (int k4 = 0; k4 < KX / 4; ++k4) {
-                const int4 q = r4[k4];
-                v[4 * k4 + 0] = (T)q.x * iq;
-                v[4 * k4 + 1] = (T)q.y * iq;
-                v[4 * k4 + 2] = (T)q.z * iq;
-                v[4 * k4 + 3] = (T)q.w * iq;
-            }
-        } else if (use_stage) {
-            // window cells to weight units: into the staging copy, else in place
-            for (int c = lane; c < L; c += 32) stage[padc(c)] = wget(row + c, iq);
-        } else if (sizeof(T) == 4) {
-            for (int c = lane; c < L; c += 32) row[c] = wget(row + c, iq);
-        }
+        if (use_stage)
+            for (int c = lane; c < L; c += 32) stage[padc(c)] = row[c];
         __syncwarp();
+        const double *from = use_stage ? stage : row;
         if (exact) {
-            solve_row_x_exact<T, KX>(direct ? nullptr : (use_stage ? stage : row), lane, v,
-                                     use_stage && !direct, sh, sl);
+            solve_row_x_exact<double, KX>(from, lane, v, use_stage, kXScale64, 0.0);
             per = KX;
             base = lane * KX;
         } else {
-            solve_row_x<T, KX>(use_stage ? stage : row, L, full, lane, v, per, base, use_stage, sh, sl);
+            solve_row_x<KX>(from, L, full, lane, v, per, base, use_stage);
         }
         __syncwarp();
-        // v * 0 is 0 for finite values and NaN otherwise
-        T chk = T(0);
-        T *dp = dst_row + base;
-        const bool inside = per == KX && base >= D && base + KX <= D + TXe;
-        if (sizeof(T) == 4 && KX % 4 == 0 && inside && ((reinterpret_cast<uintptr_t>(dp) & 15) == 0)) {
-#pragma unroll
-            for (int k = 0; k < KX; k += 4) {
-                float4 q;
-                q.x = (float)v[k];
-                q.y = (float)v[k + 1];
-                q.z = (float)v[k + 2];
-                q.w = (float)v[k + 3];
-                *reinterpret_cast<float4 *>(dp + k) = q;
-            }
-#pragma unroll
-            for (int k = 0; k < KX; ++k) chk = fma(v[k], T(0), chk);
-            if (sizeof(T) == 4)
-#pragma unroll
-                for (int k = 0; k < KX; ++k) om = fmaxf(om, fabsf((float)v[k]));
-            if (want_part) {
-                // keep s for the column sums: 16-byte stores (lanes 8 words apart: two-way bank
-                // conflicts instead of the eight-way of word stores) when the row start allows
-                if ((reinterpret_cast<uintptr_t>(row) & 15) == 0) {
-#pragma unroll
-                    for (int k = 0; k < KX; k += 4) {
-                        float4 q;
-                        q.x = (float)v[k];
-                        q.y = (float)v[k + 1];
-                        q.z = (float)v[k + 2];
-                        q.w = (float)v[k + 3];
-                        *reinterpret_cast<float4 *>(row + base + k) = q;
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < KX; ++k) row[base + k] = v[k];
-                }
-            }
-        } else if (!(exact && (base + KX <= D || base >= D + TXe))) {
+        double chk = 0.0;   // v * 0 is 0 for finite values and NaN otherwise
+        if (!(exact && (base + KX <= D || base >= D + TXe))) {
             // (lanes whose chunk lies in the halo store nothing)
 #pragma unroll
             for (int k = 0; k < KX; ++k) {
                 const int c = base + k;
                 if (k < per && c >= D && c < D + TXe) {
                     dst_row[c] = v[k];
-                    chk = fma(v[k], T(0), chk);
-                    om = fmaxf(om, fabsf((float)v[k]));
+                    chk = fma(v[k], 0.0, chk);
                     if (want_part) row[c] = v[k];   // keep s for the column sums
                 }
             }
         }
-        bad |= chk != T(0);
+        bad |= chk != 0.0;
     }
 }
 
@@ -630,7 +573,6 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
     W.own_c1 = G + D + TXe;
     W.np = np;
     W.nx = nx;
-    W.G = G;
     W.full = full;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
 
@@ -664,14 +606,9 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         s_omax = 0;
         {
             s_win.WW = W.WW;
-            s_win.WH = W.WH;
-            s_win.G = G;
-            s_win.WP0 = W.WP0;
             s_win.own_c0 = full ? 0 : W.own_c0;
             s_win.own_c1 = full ? W.WW : W.own_c1;
-            s_win.np = np;
             s_win.nx = nx;
-            s_win.edge = (P0 == 0 ? 1 : 0) | (P0 + TPe == np ? 2 : 0);
         }
     }
     double al = g.alpha0, be = g.beta0, M = g.m0, phi = g.phi0;
@@ -848,6 +785,8 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         }
     __syncthreads();   // the zeroed window, the row table, the pivots, the groups' rows
 
+    const int edge = (P0 == 0 ? 1 : 0) | (P0 + TPe == np ? 2 : 0);   // the open edges the tile owns: below, above
+
     // ---- walk the source columns
     if constexpr (sizeof(T) == 4) {
         // FP32: items of (pair of adjacent columns, segment of rows)
@@ -865,7 +804,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         K.lim = W.WH * W.ws * 4;
         K.WW = W.WW;
         K.WP0 = W.WP0;
-        K.edge = (P0 == 0 ? 1 : 0) | (P0 + TPe == np ? 2 : 0);
+        K.edge = edge;
         // kept in registers: rebuilt from the arguments at every use they cost 20 of 200 instructions a row
         K.ws4 = opaque(K.ws4);
         K.lim = opaque(K.lim);
@@ -911,7 +850,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
         K.lim = W.WH * W.ws;
         K.WW = W.WW;
         K.WP0 = W.WP0;
-        K.edge = (P0 == 0 ? 1 : 0) | (P0 + TPe == np ? 2 : 0);
+        K.edge = edge;
         const int nw = (wcol + 31) >> 5;
         for (int wi = warp; wi < nw * nseg; wi += nwarps) {
             const int sg = wi / nw, q = (wi - sg * nw) * 32 + lane, ic = ia + q;
@@ -930,7 +869,6 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
 
     // ---- guard rows beyond an open momentum edge that the tile owns: lost weight of the own columns. Where tiles are
     // lower than the guard, other tiles' windows reach past the mesh too; what lands there is the owner's to count
-    const int edge = (P0 == 0 ? 1 : 0) | (P0 + TPe == np ? 2 : 0);
     for (int k = 0; k < 2 * Gp; ++k) {   // the rows below the tile, then those above it
         if (!(edge & (k < Gp ? 1 : 2))) continue;
         const T *row = win + (size_t)(k < Gp ? k : TPe + k) * W.ws;
@@ -980,13 +918,12 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T> &A, const int tile
                                         sh, sl, iq, om, bad);
         } else {
             const int L = full ? nx : TXe + 2 * D;
-            const T sh = T(-6) * T(-0.26794919243112270647), sl = T(0);
             if (L <= 256)
-                gal_rows<T, 8>(win, W, A.dst, L, full, D, G, Gp, TXe, TPe, P0, X0, nx, want_part, warp, nwarps, lane,
-                               bad, gcol, GRows<T>::value * blockDim.x, sh, sl, iq, om);
+                solve_rows_f64<8>(win, W, A.dst, L, full, D, G, Gp, TXe, TPe, P0, X0, nx, want_part, warp, nwarps, lane,
+                                  bad, gcol, GRows<T>::value * blockDim.x);
             else
-                gal_rows<T, kXBig>(win, W, A.dst, L, full, D, G, Gp, TXe, TPe, P0, X0, nx, want_part, warp, nwarps,
-                                   lane, bad, gcol, GRows<T>::value * blockDim.x, sh, sl, iq, om);
+                solve_rows_f64<kXBig>(win, W, A.dst, L, full, D, G, Gp, TXe, TPe, P0, X0, nx, want_part, warp, nwarps,
+                                      lane, bad, gcol, GRows<T>::value * blockDim.x);
         }
     } else {
         // no solve: the deposit is the new state (its max|w| sets the next step's window scale)

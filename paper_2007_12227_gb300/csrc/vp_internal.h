@@ -101,10 +101,8 @@ struct FusedArgs {
     T *dst;
     const ColEntry<T> *col;
     const RowEntry<T> *row;
-    const RowBound *rowb;
-    const double *vcb;
-    const float4 *rowbf;    // FP32 copy of rowb: u, v, y (tile bounds)
-    const float2 *vcbf;     // FP32 copy of vcb
+    const float4 *rowbf;    // u, v, y of the rows in FP32 (tile bounds)
+    const float2 *vcbf;     // per 32-column block: min, max of the column part of dv, in FP32
     const double *state;
     const double *piv;      // Thomas pivots of tridiag(1/6, 2/3, 1/6)
     const double *sigma;    // column sums of Lambda_p^{-1} (FEL partial sums in Galerkin mode)
@@ -127,7 +125,7 @@ struct FusedArgs {
     int4 *tile_src;
     // end of the step in the same launch: every CTA takes a ticket after its tile's partial sums
     // are visible; the CTA that draws the last one updates the FEL field from all partials (or
-    // counts the step) and resets the counter. NULL: the caller finishes the step (batches).
+    // counts the step) and resets the counter.
     int *ticket;
     double *hist;           // FEL field history ring (hist_cap steps)
     int hist_cap;

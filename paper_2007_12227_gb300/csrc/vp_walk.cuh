@@ -104,13 +104,11 @@ __device__ __forceinline__ float4 lds_f4(unsigned a)
 
 // the tile's window as the walk's rare paths need it (in shared memory: no registers in the common path)
 struct WalkWin {
-    int WW, WH, G;           // window width, height, column guard band
-    int WP0;                 // grid row of window row 0
+    int WW;                  // window width
     int own_c0, own_c1;      // the columns whose lost weight the tile counts
-    int np, nx;
+    int nx;
     int wrap;                // the tile walks a whole period of source columns: first window column of the images that
                              // their nodes land at; else -1
-    int edge;                // the tile owns the first (1), the last (2) mesh row: it counts the weight lost there
 };
 
 // Weight of a row's cells a (window columns ca ..) and b (cb ..) that the tile counts as lost, countA, countB: the
@@ -185,7 +183,7 @@ struct Walk32 {
     unsigned win;
     int ws4, lim;          // bytes of a window row, of the window
     int WW, WP0;
-    int edge;              // as in WalkWin
+    int edge;              // the open edges the tile owns (1: the first mesh row, 2: the last): it counts the weight lost there
 };
 
 // One row of a pair's rings into the window. Rows outside the window belong to other tiles: they are clamped
@@ -292,6 +290,7 @@ __device__ __forceinline__ void forward_far(const char *pA, const char *pB, unsi
                                             float ncp, int na, unsigned gc, unsigned gs, f2_t &uv)
 {
     constexpr int kFly = 16, kRows = kHalo32 + kC32;
+    static_assert(kHalo32 <= kFly, "the loads of the look-ahead above the top row fit those in flight");
     f2_t x[kFly], gv = 0ull;
 #pragma unroll
     for (int k = 0; k < kFly; ++k) x[k] = load_pair<VEC>(pA, pB, pitch, k);
@@ -326,7 +325,6 @@ __device__ __forceinline__ void walk_pair(const Walk32 &K, const ColEntry<float>
     constexpr int N = BASIS == VP_BASIS_TENT ? 2 : 4;
     constexpr int LO = BASIS == VP_BASIS_TENT ? 0 : -1;
     constexpr int kBias = 0x4B400000;   // bits of 1.5 * 2^23
-    static_assert(kHalo32 <= kC32, "the look-ahead above the top row fits the column buffer");
     // sine term: al sin(a + y) + be cos(a + y) = cy (al sa + be ca) + sy (al ca - be sa)
     const float PA = al * eA.sa + be * eA.ca, QA = al * eA.ca - be * eA.sa;
     const float PB = al * eB.sa + be * eB.ca, QB = al * eB.ca - be * eB.sa;
