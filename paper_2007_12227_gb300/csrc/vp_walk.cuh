@@ -147,9 +147,9 @@ __device__ __forceinline__ int fold_col(const WalkWin *W, int m)
 {
     if (W->wrap >= 0) {
         m = (m - W->wrap) % W->nx;
-        return min(W->wrap + (m < 0 ? m + W->nx : m), W->WW - N);
+        m += W->wrap + (m < 0 ? W->nx : 0);
     }
-    return m < 0 ? 0 : W->WW - N;
+    return max(0, min(m, W->WW - N));
 }
 
 // One pair's state. The integer displacement of a node is the low mantissa bits of (fraction + 1.5 2^23)
