@@ -24,10 +24,10 @@
 //     row; when the ring moves one row, the row that leaves it is added to the
 //     window with N shared-memory atomics.
 // Contributions outside the window belong to other tiles, except rows beyond
-// the open momentum edge, which are counted as lost by the tile owning the
-// column. Finally each warp takes window rows, solves Lambda_x along them
-// (first-order recurrences over per-lane chunks, combined across lanes by a warp
-// scan, or on windowed rows by the carries of the neighbouring chunks), and the
+// an open momentum edge, which are counted as lost by the tile that owns the edge
+// row in that column. Finally each warp takes window rows, solves Lambda_x along them
+// (first-order recurrences over per-lane chunks; a lane's carry comes from the chunks
+// next to it, in FP64 rows of other lengths from a warp scan), and the
 // tile is stored once.
 #include <math.h>
 
@@ -1327,7 +1327,7 @@ int fused_batch_blocks_per_sm(int basis, int projection, size_t smem, int thread
 // and the anticausal u_i = y_i + z u_{i+1} (z = sqrt(3) - 2) run chunk-locally from zero; a
 // block-wide scan of the pairs (z^len, zero-start end value) gives each chunk its exact carry,
 // and the periodic closure adds z^{i+1} y_{-1} with y_{-1} = E / (1 - z^L), E the zero-start
-// value at L - 1 (anticausal: z^{L-i} u_L with u_L = S / (1 - z^L)), as the whole-period tiles
+// value at L - 1 (anticausal: z^{L-i} u_L with u_L = S / (1 - z^L)), as FP64 whole-period tiles
 // do within a warp. Nothing is truncated. A whole chunk takes its carry and closure as one term,
 // z^{k+1} (carry + z^base y_{-1}), with the powers of z as compile-time constants.
 // The row sits in shared memory with element c at c + V (c / (32 V)), V the elements of 16
@@ -1551,7 +1551,9 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1)
     // FP64 row's operations)
     const T zbase = base < 128 ? zpow<T>(base) : T(0), zend = nx - base - len < 128 ? zpow<T>(nx - base - len) : T(0);
     const T closure = nx < 128 ? T(1) / (T(1) - zpow<T>(nx)) : T(1);
-    // a chunk lies in one tile when the tile width is a multiple of the chunk
+    // A chunk lies in one tile when the tile width is a multiple of the chunk. The default FP32 width without an x
+    // halo, 240, is not: maxima element by element cost the pass 38 instructions a node for 28.6, 0.112 ms for
+    // 0.097 (8192 x 8192), and the tile kernel gains more by the width (the autotuner's pick among 224, 240 and 256)
     const bool one_tile = tx % K == 0;
 
     // zeros past the row end in every buffer (read with the last chunks, never stored)

@@ -329,7 +329,9 @@ __device__ __forceinline__ void walk_pair(const Walk32 &K, const ColEntry<float>
     const float PA = al * eA.sa + be * eA.ca, QA = al * eA.ca - be * eA.sa;
     const float PB = al * eB.sa + be * eB.ca, QB = al * eB.ca - be * eB.sa;
     const f2_t cv1 = f2_pack(KV * PA, KV * PB), cv2 = f2_pack(KV * QA, KV * QB);
-    const f2_t KR = f2_dup(KV != 0.f ? KU / KV : 0.f);   // both are multiples of the same step
+    // KU s from KV s: both are multiples of the same step. (The quotient's rounding, 6e-8 of the kick along x, is
+    // of the size of KU's own in FP32; it saves two pairs of column constants)
+    const f2_t KR = f2_dup(KV != 0.f ? KU / KV : 0.f);
     // window column / row of the first tap = key + base (+ the row index)
     const int buA = colrel + eA.ui - kBias + LO, buB = colrel + 1 + eB.ui - kBias + LO;
     const int bvA = eA.vi - kBias + LO - K.WP0, bvB = eB.vi - kBias + LO - K.WP0;
