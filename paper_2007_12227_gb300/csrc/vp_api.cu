@@ -206,8 +206,12 @@ vp_status make_plan(const vp_grid *grid, int32_t basis, const vp_pusher *pu, con
         const int halo = P->galerkin && !P->xpass ? fused_halo(opts->precision) : 0;
         const int R = basis == VP_BASIS_TENT ? 1 : 2;
         const int G = P->G, Gp = P->Gp;
-        // FP32 by default: 256 columns with the halo and the guard (the x pass on a mesh that is no wider: 224)
-        const int width32 = halo ? 208 : (P->xpass && grid->nx <= 240 + 2 * G ? 224 : 240);
+        // FP32 by default: 256 columns with the halo and the guard. With the x pass 224, a multiple of its threads' 32
+        // nodes (a step of 357 x 300 23.1 us for 25.8 with 240, of 4096 x 4096 134.9 for 141.0, of 8192 x 8192 492 for
+        // 495), but 240 where only that takes one wave of tiles (2048 x 2048: 44.6 us, 52.2 with 224)
+        auto tiles64 = [&](int w) { return (long)((grid->nx + w - 1) / w) * ((grid->np + 63) / 64); };
+        const bool one_wave = grid->nx > 240 + 2 * G && tiles64(240) <= kSlots && tiles64(224) > kSlots;
+        const int width32 = halo ? 208 : (P->xpass && !one_wave ? 224 : 240);
         ftx = opts->tile_x ? opts->tile_x : (opts->precision == VP_FP64 ? 112 : width32);
         ftp = opts->tile_p ? opts->tile_p : 64;
         bool full = false;

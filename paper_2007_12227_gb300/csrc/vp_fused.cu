@@ -1551,9 +1551,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1)
     // FP64 row's operations)
     const T zbase = base < 128 ? zpow<T>(base) : T(0), zend = nx - base - len < 128 ? zpow<T>(nx - base - len) : T(0);
     const T closure = nx < 128 ? T(1) / (T(1) - zpow<T>(nx)) : T(1);
-    // A chunk lies in one tile when the tile width is a multiple of the chunk. The default FP32 width without an x
-    // halo, 240, is not: maxima element by element cost the pass 38 instructions a node for 28.6, 0.112 ms for
-    // 0.097 (8192 x 8192), and the tile kernel gains more by the width (the autotuner's pick among 224, 240 and 256)
+    // A chunk lies in one tile when the tile width is a multiple of the chunk, as the planner's 224 is; for other widths
+    // the maxima are found element by element (240: 38 instructions a node for 28, 0.112 ms for 0.095, 8192 x 8192)
     const bool one_tile = tx % K == 0;
 
     // zeros past the row end in every buffer (read with the last chunks, never stored)

@@ -90,3 +90,9 @@ def test_wide_tiles_are_planned_at_one_block_an_sm(nx, np_, precision, tile_x):
     """The default height gives every SM one such tile: fewer than 152 tiles, and more than half of that."""
     plan = run(nx, np_, precision, FUSED, (tile_x, 0), steps=2)
     assert 76 < plan["ntiles_x"] * plan["ntiles_p"] <= 152
+
+
+@pytest.mark.parametrize("nx,np_,tile_x", [(300, 300, 224), (1000, 200, 224), (2048, 2048, 240)])
+def test_separate_x_pass_fp32_default_width(nx, np_, tile_x):
+    """A multiple of the row pass's 32 nodes, or what takes one wave of tiles."""
+    assert run(nx, np_, I.FP32, XP, steps=1)["tile_x"] == tile_x
